@@ -148,6 +148,31 @@ hz_status launch_sweep_cluster_f64(int P, const SweepArgs& a, int L, cudaStream_
 // shape fits.
 hz_status launch_sweep_cband(int P, const SweepArgs& a, int L, cudaStream_t st);
 
+// Sweep by element tiles (hz_sweep_tile.cuh): subdomains of at most 32 x 32
+// elements, degree 1..5 (FP64: 1..4, with a source 1..3), eta = 0, cold start.
+// a.ty_force: 1 = one element per tile, 2 = two, paired (FP32, P <= 4, even
+// sub_ny), 0 = by size (tile_shape).  *warps: warps per subdomain, 0 for a
+// cluster.  HZ_ERR_UNSUPPORTED (nothing launched) else.
+hz_status launch_sweep_tile(bool fp32, int P, const SweepArgs& a, int count, cudaStream_t st, int* warps);
+// Shape of the tile sweep for a subdomain (1 or 2), and whether it is the
+// default kernel there (without the autotuner).  L: subdomains of the problem.
+int tile_shape(bool fp32, int P, int sxe, int sye, int L);
+bool tile_default(bool fp32, int P, int sxe, int sye, int L);
+// Largest block of a tile shape.  Registers are allocated per scheduler (a
+// quarter of the SM's 65536), so a thread has 255 of them in blocks of up to
+// 8 warps, 168 up to 12, 128 up to 16, 80 up to 24.  A tile needs 5 (with a
+// source 7) values per node and 50 to 80 registers more for coefficients,
+// addresses and temporaries.
+constexpr int tile_max_threads(bool f64, int P, int H, bool src) {
+  const int words = P * P * H * (src ? 7 : 5) * (f64 ? 2 : 1);
+  return words <= 10 ? 768 : words <= 40 ? 512 : words <= 90 ? 384 : 256;
+}
+constexpr int tile_pow2(int n) {  // smallest power of two >= n
+  int p = 1;
+  while (p < n) p *= 2;
+  return p;
+}
+
 // Launches the sweep in Real = float (fp32 = true) or double.  Returns
 // HZ_ERR_UNSUPPORTED when no compiled variant fits the subdomain.
 hz_status launch_sweep_f32(int P, const SweepArgs& a, int L, cudaStream_t st);

@@ -221,6 +221,7 @@ int sweep_variant() {
   if (std::strcmp(v, "warp") == 0) return kVariantWarp;
   if (std::strcmp(v, "cluster") == 0) return kVariantCluster;
   if (std::strcmp(v, "cband") == 0) return kVariantClusterBand;
+  if (std::strcmp(v, "tile") == 0) return kVariantTile;
   return kVariantAuto;
 }
 
@@ -265,6 +266,17 @@ hz_status launch_choice(Problem& pr, const SweepArgs& a0, Choice c, bool fp32, c
   const Geom& g = pr.g;
   const int count = sweep_count(a0, g.L);
   hz_status s = HZ_ERR_UNSUPPORTED;
+  if (c.variant == kVariantTile) {
+    int warps = 0;
+    SweepArgs a = a0;
+    a.ty_force = c.ty;  // elements per tile: 1, 2 or 0 = by size
+    s = launch_sweep_tile(fp32, g.P, a, count, st, &warps);
+    if (s == HZ_OK) {  // reported with the register-resident kernels by warps per subdomain, or as a cluster
+      pr.last_variant = warps > 0 ? kVariantWarp : kVariantClusterBand;
+      pr.last_shape = warps;
+    }
+    return s;
+  }
   if (c.variant == kVariantWarp) {
     if (!fp32) return HZ_ERR_UNSUPPORTED;
     WarpSweepArgs w{};
@@ -367,9 +379,9 @@ hz_status autotune(Problem& pr, int precision, int nt, int m_wh, cudaStream_t st
   const SweepArgs a = make_sweep_args(pr, fp32, nt, m_wh, 0.0, pr.xv.as<double>(), pr.tv.as<double>(), nullptr, nullptr);
   std::vector<Choice> cands;
   if (fp32)
-    cands = {{kVariantWarp, 1}, {kVariantWarp, 2}, {kVariantWarp, 4}, {kVariantBlock, 1}, {kVariantBlock, 2},
+    cands = {{kVariantTile, 1}, {kVariantTile, 2}, {kVariantWarp, 1}, {kVariantWarp, 2}, {kVariantWarp, 4}, {kVariantBlock, 1}, {kVariantBlock, 2},
              {kVariantCluster, 0}, {kVariantCluster, 4}, {kVariantClusterBand, 0}, {kVariantClusterBand, 8}};
-  else cands = {{kVariantBlock, 1}, {kVariantBlock, 2}, {kVariantCluster, 0}, {kVariantCluster, 4}};
+  else cands = {{kVariantTile, 1}, {kVariantBlock, 1}, {kVariantBlock, 2}, {kVariantCluster, 0}, {kVariantCluster, 4}};
   cudaEvent_t e0, e1;
   HZ_CUDA(cudaEventCreate(&e0));
   HZ_CUDA(cudaEventCreate(&e1));
@@ -519,6 +531,13 @@ hz_status sweep(Problem& pr, int precision, int nt, int m_wh, double wh_tol, con
   if (have) {
     ls = launch_choice(pr, a, ch, fp32, st);
     if (ls != HZ_OK && ls != HZ_ERR_UNSUPPORTED) return ls;
+  }
+  if (ls == HZ_ERR_UNSUPPORTED && !trial &&
+      (want == kVariantTile || (want == kVariantAuto && !std::getenv("HZ_SWEEP_WARPS") &&
+                                tile_default(fp32, g.P, g.snx, g.sny, g.L)))) {
+    ls = launch_choice(pr, a, Choice{kVariantTile, 0}, fp32, st);
+    if (ls != HZ_OK && ls != HZ_ERR_UNSUPPORTED) return ls;
+    if (ls != HZ_OK && want == kVariantTile) return fail(HZ_ERR_UNSUPPORTED, "no tile sweep shape fits");
   }
   if (ls == HZ_ERR_UNSUPPORTED && fp32 && (want == kVariantAuto || want == kVariantWarp)) {
     // HZ_SWEEP_WARPS=2|4 forces warps per subdomain of the register-resident kernel (tests)
