@@ -116,90 +116,205 @@ __global__ void rhs_kernel(const __grid_constant__ GlobalArgs a, const double* _
   b[2 * n + 1] = bi;
 }
 
+// 1 / x for finite x > 0 by Newton's iteration y <- y (2 - x y) from an FP32
+// reciprocal: each step squares the relative error (2^-22, 2^-44, below one
+// unit in the last place), four FP64 FMAs instead of a division's dozen.  The
+// FP32 values are cut out of and put back into the FP64 words by shifts (the
+// conversion instructions run at the FP64 rate).  Outside FP32's range the
+// division itself.
+__device__ __forceinline__ double recip(double x) {
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  if (hi - (937u << 20) >= (172u << 20)) return 1.0 / x;  // outside 2^-86 .. 2^86
+  const float f = __uint_as_float(((hi - (896u << 20)) << 3) | (lo >> 29));  // x cut to 23 bits
+  const unsigned q = __float_as_uint(__frcp_rn(f));
+  double y = __hiloint2double((int)((q >> 3) + (896u << 20)), (int)(q << 29));
+  y = fma(y, fma(-x, y, 1.0), y);
+  return fma(y, fma(-x, y, 1.0), y);
+}
+
 // ---- r = b - (A - i w H - w^2 M) u on the global grid (Sec. 4), FP64.
-// A u = Wy_J (Kx u)_IJ + Wx_I (Ky u)_IJ with assembled 1D rows built from the
-// reference element stiffness (one-sided at the outer boundary).
+//   A u = Wx Wy [(Kx u) / Wx + (Ky u) / Wy], the assembled 1D rows divided by
+// their lumped weights (host tables a.Kx, a.Ky by node class), so that
+//   r = b - Wx Wy [(Kx u) / Wx + (Ky u) / Wy - (w/c)^2 u] + i (w/c) Hw u,
+// the last term on the outer boundary only; both centre taps and -(w/c)^2 make
+// one coefficient of the node's own value (a.Kd by the two classes).
+// The FP64 pipe bounds it (about 1.7 FMA per clock and SM).  A thread per node
+// ran the 2P + 1 taps of the widest row class on every lane and two divisions:
+// 106 us on 769 x 769 nodes, P = 3, with the sums' second launch; 51 us now (41 us
+// is 33 FP64 instructions per node at the pipe's measured rate).  Here a thread owns the P nodes of one
+// element in one node row: the x class of a node is known at compile time, the
+// y class is uniform in the warp, so a node runs only its own taps (5 instead
+// of 7 on average at P = 3), and one reciprocal serves both divisions.  The
+// mesh's last node column has blocks of its own, a thread per node (as a
+// 33rd lane's work it cost a whole warp per row).  Blocks of four rows: more
+// of them than eight rows give, for an even load of the SMs.
+constexpr int kResRows = 4;
+struct ResNode {  // what a node adds to the two sums
+  double rr = 0.0, bb = 0.0;
+};
+// S: the node's taps including its own value's
+__device__ __forceinline__ void residual_node(int64_t n, double W, double h, double2 u, double2 S,
+                                              const double* __restrict__ b, double* __restrict__ r, ResNode& sum) {
+  double2 bn = make_double2(0.0, 0.0);
+  if (b) bn = reinterpret_cast<const double2*>(b)[n];
+  double rr = fma(-W, S.x, bn.x);
+  double ri = fma(-W, S.y, bn.y);
+  if (h != 0.0) {
+    rr = fma(-h, u.y, rr);
+    ri = fma(h, u.x, ri);
+  }
+  reinterpret_cast<double2*>(r)[n] = make_double2(rr, ri);
+  sum.rr = fma(rr, rr, fma(ri, ri, sum.rr));
+  if (b) sum.bb = fma(bn.x, bn.x, fma(bn.y, bn.y, sum.bb));
+}
+
 template <int P>
-__global__ void residual_kernel(const __grid_constant__ GlobalArgs a, const double* __restrict__ b,
-                                const double* __restrict__ u, double* __restrict__ r, double* __restrict__ part) {
-  // the assembled rows in shared memory: the lanes of a warp index them by
-  // their own node class (a per-lane index into parameter space serialises)
-  __shared__ double kx[P + 2][2 * P + 1], ky[P + 2][2 * P + 1];
-  for (int k = threadIdx.y * blockDim.x + threadIdx.x; k < (P + 2) * (2 * P + 1); k += blockDim.x * blockDim.y) {
-    kx[k / (2 * P + 1)][k % (2 * P + 1)] = a.Kx[k / (2 * P + 1)][k % (2 * P + 1)];
-    ky[k / (2 * P + 1)][k % (2 * P + 1)] = a.Ky[k / (2 * P + 1)][k % (2 * P + 1)];
-  }
-  __syncthreads();
-  const int I = blockIdx.x * blockDim.x + threadIdx.x;
-  const int J = blockIdx.y * blockDim.y + threadIdx.y;
-  double sums[2] = {0.0, 0.0};
-  if (I < a.NXg && J < a.NYg) {
-    const int64_t n = (int64_t)J * a.NXg + I;
-    const double2* u2 = reinterpret_cast<const double2*>(u);
-    // x and y: assembled rows from the host tables (node class by position
-    // in its element, first and last node of the mesh separately)
-    const int cx = (I == 0) ? P : (I == a.NXg - 1) ? P + 1 : I % P;
-    const int cy = (J == 0) ? P : (J == a.NYg - 1) ? P + 1 : J % P;
-    double sxr = 0.0, sxi = 0.0, syr = 0.0, syi = 0.0;
+__global__ void __launch_bounds__(32 * kResRows)
+    residual_kernel(const __grid_constant__ GlobalArgs a, int nbx, int nmain, const double* __restrict__ b,
+                    const double* __restrict__ u, double* __restrict__ r, double* __restrict__ part,
+                    unsigned* __restrict__ ticket, double* __restrict__ norms2) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const double2* u2 = reinterpret_cast<const double2*>(u);
+  ResNode sum;
+  if ((int)blockIdx.x < nmain) {
+    const int ex = (int)(blockIdx.x % nbx) * 32 + lane;
+    const int J = (int)(blockIdx.x / nbx) * kResRows + warp;
+    if (ex < a.nx && J < a.NYg) {
+      const int64_t n0 = (int64_t)J * a.NXg + (int64_t)ex * P;
+      double2 v[P + 1], S[P];
 #pragma unroll
-    for (int tt = -P; tt <= P; ++tt) {
-      if (I + tt >= 0 && I + tt < a.NXg) {  // taps outside the mesh have coefficient 0
-        const double2 v = __ldg(&u2[n + tt]);
-        const double cf = kx[cx][tt + P];
-        sxr = fma(cf, v.x, sxr);
-        sxi = fma(cf, v.y, sxi);
+      for (int k = 0; k <= P; ++k) v[k] = __ldg(&u2[n0 + k]);
+      // y: the element row's own nodes, and on a shared row the element below
+      const int ay = J % P;
+      const int cy = J == 0 ? P : J == a.NYg - 1 ? P + 1 : ay;
+      double t[P];
+#pragma unroll
+      for (int k = 0; k < P; ++k) {
+        t[k] = a.omega * recip(a.c[n0 + k]);
+        const double d = fma(-t[k], t[k], k == 0 && ex == 0 ? a.Kd[P][cy] : a.Kd[k][cy]);
+        S[k] = make_double2(d * v[k].x, d * v[k].y);
       }
-      if (J + tt >= 0 && J + tt < a.NYg) {
-        const double2 v = __ldg(&u2[n + (int64_t)tt * a.NXg]);
-        const double cf = ky[cy][tt + P];
-        syr = fma(cf, v.x, syr);
-        syi = fma(cf, v.y, syi);
+      auto yrow = [&](int off) {  // row J + off, 0 < |off| <= P
+        const double cf = a.Ky[cy][P + off];
+        const double2* row = u2 + n0 + (int64_t)off * a.NXg;
+#pragma unroll
+        for (int k = 0; k < P; ++k) {
+          const double2 w = __ldg(&row[k]);
+          S[k].x = fma(cf, w.x, S[k].x);
+          S[k].y = fma(cf, w.y, S[k].y);
+        }
+      };
+      if (J < a.NYg - 1) {
+#pragma unroll
+        for (int t = 0; t <= P; ++t)
+          if (t != ay) yrow(t - ay);
+      }
+      if (ay == 0 && J > 0) {
+#pragma unroll
+        for (int t = 1; t <= P; ++t) yrow(-t);
+      }
+      // x: the element's own nodes; node 0 also the element to the left
+#pragma unroll
+      for (int k = 1; k <= P; ++k) {
+        const double cf = ex > 0 ? a.Kx[0][P + k] : a.Kx[P][P + k];
+        S[0].x = fma(cf, v[k].x, S[0].x);
+        S[0].y = fma(cf, v[k].y, S[0].y);
+      }
+      if (ex > 0) {
+#pragma unroll
+        for (int k = 1; k <= P; ++k) {
+          const double2 w = __ldg(&u2[n0 - k]);
+          S[0].x = fma(a.Kx[0][P - k], w.x, S[0].x);
+          S[0].y = fma(a.Kx[0][P - k], w.y, S[0].y);
+        }
+      }
+#pragma unroll
+      for (int q = 1; q < P; ++q)
+#pragma unroll
+        for (int k = 0; k <= P; ++k) {
+          if (k == q) continue;
+          S[q].x = fma(a.Kx[q][P + k - q], v[k].x, S[q].x);
+          S[q].y = fma(a.Kx[q][P + k - q], v[k].y, S[q].y);
+        }
+      const double Wy = a.Wyg[J];
+      const bool yb = J == 0 || J == a.NYg - 1;
+#pragma unroll
+      for (int q = 0; q < P; ++q) {
+        const double Wx = a.Wxg[ex * P + q];
+        double h = 0.0;
+        if (yb || (q == 0 && ex == 0)) h = t[q] * ((yb ? Wx : 0.0) + (q == 0 && ex == 0 ? Wy : 0.0));
+        residual_node(n0 + q, Wx * Wy, h, v[q], S[q], b, r, sum);
       }
     }
-    const double Wx = a.Wxg[I], Wy = a.Wyg[J];
-    const double Aur = Wy * sxr + Wx * syr;
-    const double Aui = Wy * sxi + Wx * syi;
-    const double c = a.c[n];
-    const double M = Wx * Wy / (c * c);
-    const double H = (((J == 0 || J == a.NYg - 1) ? Wx : 0.0) + ((I == 0 || I == a.NXg - 1) ? Wy : 0.0)) / c;
-    const double2 un = u2[n];
-    const double w = a.omega;
-    // K u = A u - i w H u - w^2 M u
-    const double Kur = Aur + w * H * un.y - w * w * M * un.x;
-    const double Kui = Aui - w * H * un.x - w * w * M * un.y;
-    double br = 0.0, bi = 0.0;
-    if (b) { br = b[2 * n]; bi = b[2 * n + 1]; }
-    const double rr = br - Kur, ri = bi - Kui;
-    r[2 * n] = rr;
-    r[2 * n + 1] = ri;
-    sums[0] = rr * rr + ri * ri;
-    sums[1] = br * br + bi * bi;
+  } else {
+    const int J = ((int)blockIdx.x - nmain) * 32 * kResRows + (int)threadIdx.x;
+    if (J < a.NYg) {
+      const int I = a.NXg - 1;
+      const int64_t n = (int64_t)J * a.NXg + I;
+      const int cy = J == 0 ? P : J == a.NYg - 1 ? P + 1 : J % P;
+      const double t = a.omega * recip(a.c[n]), d = fma(-t, t, a.Kd[P + 1][cy]);
+      const double2 un = u2[n];
+      double2 S = make_double2(d * un.x, d * un.y);
+      for (int k = -P; k <= P; ++k) {
+        if (k == 0) continue;
+        if (J + k >= 0 && J + k < a.NYg) {  // taps outside the row's class have coefficient 0
+          const double2 w = __ldg(&u2[n + (int64_t)k * a.NXg]);
+          S.x = fma(a.Ky[cy][P + k], w.x, S.x);
+          S.y = fma(a.Ky[cy][P + k], w.y, S.y);
+        }
+        if (k < 0) {
+          const double2 w = __ldg(&u2[n + k]);
+          S.x = fma(a.Kx[P + 1][P + k], w.x, S.x);
+          S.y = fma(a.Kx[P + 1][P + k], w.y, S.y);
+        }
+      }
+      const double Wx = a.Wxg[I], Wy = a.Wyg[J];
+      residual_node(n, Wx * Wy, t * (Wy + (J == 0 || J == a.NYg - 1 ? Wx : 0.0)), un, S, b, r, sum);
+    }
   }
-  // flatten the 2D block for the reduction
-  __shared__ double out[2];
-  const int tid = threadIdx.y * blockDim.x + threadIdx.x;
-  {
-    __shared__ double sh[2][32];
-    const int lane = tid & 31, warp = tid >> 5;
-    const int nw = (blockDim.x * blockDim.y + 31) >> 5;
-    for (int k = 0; k < 2; ++k) {
-      double x = warp_sum(sums[k]);
-      if (lane == 0) sh[k][warp] = x;
+  if (!norms2) return;
+  // the block's sums in a fixed order, one warp per sum (a warp reduction in
+  // every warp is as many FP64 instructions as the taps of half a node)
+  constexpr int kT = 32 * kResRows;
+  __shared__ double sh[2][kT];
+  __shared__ bool last;
+  sh[0][threadIdx.x] = sum.rr;
+  sh[1][threadIdx.x] = sum.bb;
+  __syncthreads();
+  if (warp < 2) {
+    double x = 0.0;
+    if (warp == 0 || b) {
+#pragma unroll
+      for (int k = 0; k < kResRows; ++k) x += sh[warp][32 * k + lane];
+      x = warp_sum(x);
     }
-    __syncthreads();
-    if (warp == 0) {
-      for (int k = 0; k < 2; ++k) {
-        double x = (lane < nw) ? sh[k][lane] : 0.0;
-        x = warp_sum(x);
-        if (lane == 0) out[k] = x;
-      }
+    if (lane == 0) {
+      part[2 * (int64_t)blockIdx.x + warp] = x;
+      __threadfence();
     }
-    __syncthreads();
   }
-  if (tid == 0) {
-    const int blk = blockIdx.y * gridDim.x + blockIdx.x;
-    part[2 * blk] = out[0];
-    part[2 * blk + 1] = out[1];
+  // the last block to finish adds the blocks' sums, in block order (the ticket
+  // wraps to zero for the next call)
+  __syncthreads();
+  if (threadIdx.x == 0) last = atomicInc(ticket, gridDim.x - 1) == gridDim.x - 1;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  double x0 = 0.0, x1 = 0.0;
+  for (int k = threadIdx.x; k < (int)gridDim.x; k += kT) {
+    const double2 p = __ldcg(reinterpret_cast<const double2*>(part) + k);
+    x0 += p.x;
+    x1 += p.y;
+  }
+  sh[0][threadIdx.x] = x0;
+  sh[1][threadIdx.x] = x1;
+  __syncthreads();
+  if (warp < 2) {
+    double x = 0.0;
+#pragma unroll
+    for (int k = 0; k < kResRows; ++k) x += sh[warp][32 * k + lane];
+    x = warp_sum(x);
+    if (lane == 0) norms2[warp] = x;
   }
 }
 
@@ -402,15 +517,16 @@ int grid_for(int64_t n, int threads) {
   return (int)g;
 }
 
+// Blocks of the residual kernel: element columns x node rows, then the last node column.
+int residual_main_blocks(const GlobalArgs& a) { return (a.nx + 31) / 32 * ((a.NYg + kResRows - 1) / kResRows); }
+
 template <int P>
 hz_status launch_residual_P(const GlobalArgs& a, const double* b, const double* u, double* r, double* part,
-                            int* nb, cudaStream_t st) {
-  dim3 blk(32, 8);
-  dim3 grd((a.NXg + 31) / 32, (a.NYg + 7) / 8);
-  residual_kernel<P><<<grd, blk, 0, st>>>(a, b, u, r, part);
+                            unsigned* ticket, double* norms2, cudaStream_t st) {
+  residual_kernel<P><<<residual_blocks(a), 32 * kResRows, 0, st>>>(a, (a.nx + 31) / 32, residual_main_blocks(a), b, u,
+                                                                   r, part, ticket, norms2);
   note_launch();
   HZ_CUDA(cudaGetLastError());
-  *nb = (int)(grd.x * grd.y);
   return HZ_OK;
 }
 
@@ -433,18 +549,20 @@ hz_status launch_rhs(const GlobalArgs& a, const double* f, const double* gb, dou
   return HZ_OK;
 }
 
-int residual_blocks(const GlobalArgs& a) { return ((a.NXg + 31) / 32) * ((a.NYg + 7) / 8); }
+int residual_blocks(const GlobalArgs& a) {
+  return residual_main_blocks(a) + (a.NYg + 32 * kResRows - 1) / (32 * kResRows);
+}
 
 hz_status launch_residual(const GlobalArgs& a, const double* b, const double* u, double* r, double* part,
-                          int* nblocks, cudaStream_t st) {
+                          unsigned* ticket, double* norms2, cudaStream_t st) {
   switch (a.P) {
-    case 1: return launch_residual_P<1>(a, b, u, r, part, nblocks, st);
-    case 2: return launch_residual_P<2>(a, b, u, r, part, nblocks, st);
-    case 3: return launch_residual_P<3>(a, b, u, r, part, nblocks, st);
-    case 4: return launch_residual_P<4>(a, b, u, r, part, nblocks, st);
-    case 5: return launch_residual_P<5>(a, b, u, r, part, nblocks, st);
-    case 6: return launch_residual_P<6>(a, b, u, r, part, nblocks, st);
-    case 7: return launch_residual_P<7>(a, b, u, r, part, nblocks, st);
+    case 1: return launch_residual_P<1>(a, b, u, r, part, ticket, norms2, st);
+    case 2: return launch_residual_P<2>(a, b, u, r, part, ticket, norms2, st);
+    case 3: return launch_residual_P<3>(a, b, u, r, part, ticket, norms2, st);
+    case 4: return launch_residual_P<4>(a, b, u, r, part, ticket, norms2, st);
+    case 5: return launch_residual_P<5>(a, b, u, r, part, ticket, norms2, st);
+    case 6: return launch_residual_P<6>(a, b, u, r, part, ticket, norms2, st);
+    case 7: return launch_residual_P<7>(a, b, u, r, part, ticket, norms2, st);
     default: return fail(HZ_ERR_UNSUPPORTED, "degree outside 1..7");
   }
 }

@@ -207,20 +207,22 @@ struct GlobalArgs {
   double w[kMaxP + 1];
   // assembled 1D stiffness rows by node class (class a = node a of an
   // element, 0 < a < P or a = 0 with elements on both sides; class P: first
-  // node of the mesh; class P+1: last node), taps -P..P, scaled by 2/hx (Kx)
-  // or 2/hy (Ky); built on the host
+  // node of the mesh; class P+1: last node), taps -P..P, divided by the row's
+  // lumped weight; built on the host
   double Kx[kMaxP + 2][2 * kMaxP + 1];
   double Ky[kMaxP + 2][2 * kMaxP + 1];
+  double Kd[kMaxP + 2][kMaxP + 2];  // the centre taps' sum by x and y class
   const double* c;
   const double* Wxg;
   const double* Wyg;
 };
 // b = (f, phi) + <g, phi>; f: n complex; gb: boundary S,E,N,W complex.
 hz_status launch_rhs(const GlobalArgs& a, const double* f, const double* gb, double* b, cudaStream_t st);
-// r = b - K u (b may be null); partial sums of |r|^2, |b|^2 per block into part (2 per block);
-// returns the number of blocks used through *nblocks.
+// r = b - K u (b may be null); with norms2 also |r|^2, |b|^2 (device memory),
+// through part (2 doubles per block, residual_blocks) and *ticket (device
+// memory, zero before the first call; every call leaves it zero).
 hz_status launch_residual(const GlobalArgs& a, const double* b, const double* u, double* r, double* part,
-                          int* nblocks, cudaStream_t st);
+                          unsigned* ticket, double* norms2, cudaStream_t st);
 int residual_blocks(const GlobalArgs& a);
 // out[k] = sum over blocks of part[blocks][k] for k < width, in fixed order.
 hz_status launch_reduce_partials(const double* part, int nblocks, int width, double* out, cudaStream_t st);

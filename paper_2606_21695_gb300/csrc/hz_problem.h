@@ -48,7 +48,7 @@ struct hz_problem_s {
   // leapfrog coefficients for prepared_nt
   hz::DevBuf beta64, alpha64, beta32, alpha32, kedge, tab64, tab32;
   // solver workspace
-  hz::DevBuf bvec, rvec, uvec, usub, gv, xv, tv, V, part, small, flags, hcol;
+  hz::DevBuf bvec, rvec, uvec, usub, gv, xv, tv, V, part, small, flags, hcol, ticket;
   hz::DevBuf uwarm;  // subdomain solutions carried between sweeps (opts.wh_warm)
   hz::DevBuf Vg, Zg;  // global Krylov and preconditioned vectors of the FGMRES refinement
   hz::HostBuf hsmall, hcol_host;

@@ -106,7 +106,7 @@ static GlobalArgs global_args(const Problem& pr) {
   a.hy2 = g.hy / 2.0;
   for (size_t k = 0; k < g.Kref.size(); ++k) a.Kref[k] = g.Kref[k];
   for (int k = 0; k <= g.P; ++k) a.w[k] = g.w[k];
-  // assembled rows: class c < P is an element's node c (c = 0: also node P of
+  // assembled rows over their lumped weights: class c < P is an element's node c (c = 0: also node P of
   // the element to the left); class P the mesh's first node (own element
   // only), class P+1 its last node (left element only)
   const int P = g.P;
@@ -118,9 +118,12 @@ static GlobalArgs global_args(const Problem& pr) {
       const int bb = ax + tt;
       if (own && bb >= 0 && bb <= P) v += g.Kref[(size_t)ax * (P + 1) + bb];
       if (left && tt <= 0) v += g.Kref[(size_t)P * (P + 1) + (tt + P)];
-      a.Kx[c][tt + P] = v * a.kxs;
-      a.Ky[c][tt + P] = v * a.kys;
+      const double w = (own ? g.w[ax] : 0.0) + (left ? g.w[P] : 0.0);
+      a.Kx[c][tt + P] = v * a.kxs / (w * a.hx2);
+      a.Ky[c][tt + P] = v * a.kys / (w * a.hy2);
     }
+  for (int cx = 0; cx < P + 2; ++cx)
+    for (int cy = 0; cy < P + 2; ++cy) a.Kd[cx][cy] = a.Kx[cx][P] + a.Ky[cy][P];
   a.c = pr.c.as<double>();
   a.Wxg = pr.Wxg.as<double>();
   a.Wyg = pr.Wyg.as<double>();
@@ -610,12 +613,13 @@ hz_status residual(Problem& pr, const double* b, const double* u, double* r, dou
     return HZ_OK;
   }
   const GlobalArgs a = global_args(pr);
-  const int nb = residual_blocks(a);
-  HZ_TRY(pr.part.ensure((size_t)std::max(nb, 1) * 2 * sizeof(double)));
-  int used = 0;
-  HZ_TRY(launch_residual(a, b, u, r, pr.part.as<double>(), &used, st));
-  if (norms2_dev) HZ_TRY(launch_reduce_partials(pr.part.as<double>(), used, 2, norms2_dev, st));
-  return HZ_OK;
+  HZ_TRY(pr.part.ensure((size_t)residual_blocks(a) * 2 * sizeof(double)));
+  if (!pr.ticket.ptr) {
+    HZ_TRY(pr.ticket.ensure(16));
+    HZ_CUDA(cudaMemset(pr.ticket.ptr, 0, 16));
+    HZ_UPLOADS_DONE();
+  }
+  return launch_residual(a, b, u, r, pr.part.as<double>(), static_cast<unsigned*>(pr.ticket.ptr), norms2_dev, st);
 }
 
 hz_status rhs(Problem& pr, double* b, cudaStream_t st) {
