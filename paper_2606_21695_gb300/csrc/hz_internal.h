@@ -251,6 +251,13 @@ inline hz_status launch_sweep_mapped(bool fp32, int P, const MappedSweepArgs& a,
   return fp32 ? launch_sweep_mapped_f32(P, a, L, st) : launch_sweep_mapped_f64(P, a, L, st);
 }
 
+// The FP32 mapped sweep with one element per thread (hz_sweep_mapped_tile.cuh,
+// degree 1..4, at most 32 element columns and 256 tiles); HZ_ERR_UNSUPPORTED
+// (nothing launched) else.
+hz_status launch_sweep_mapped_tile(int P, const MappedSweepArgs& a, int L, cudaStream_t st);
+// Whether it is the default there (L: subdomains of the problem).
+bool mapped_tile_default(int P, int snx, int sny, int L);
+
 struct MappedGlobalArgs {
   int NXg, NYg, nx, ny, P;
   double omega;

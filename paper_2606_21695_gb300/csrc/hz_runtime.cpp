@@ -465,7 +465,14 @@ hz_status sweep(Problem& pr, int precision, int nt, int m_wh, double wh_tol, con
     ma.snx = g.snx;
     ma.sny = g.sny;
     for (size_t k = 0; k < pr.mapped_D.size(); ++k) ma.D[k] = pr.mapped_D[k];
-    HZ_TRY(launch_sweep_mapped(fp32, g.P, ma, count, st));
+    // HZ_SWEEP_VARIANT=block / tile force the one-thread-per-node / -element kernel (tests)
+    hz_status ms = HZ_ERR_UNSUPPORTED;
+    const int mv = sweep_variant();
+    if (fp32 && (mv == kVariantTile || (mv != kVariantBlock && mapped_tile_default(g.P, g.snx, g.sny, g.L)))) {
+      ms = launch_sweep_mapped_tile(g.P, ma, count, st);
+      if (ms != HZ_OK && (ms != HZ_ERR_UNSUPPORTED || mv == kVariantTile)) return ms;
+    }
+    if (ms != HZ_OK) HZ_TRY(launch_sweep_mapped(fp32, g.P, ma, count, st));
     pr.last_variant = kVariantMapped;
     pr.last_shape = 0;
     if (e1) HZ_CUDA(cudaEventRecord(e1, st));

@@ -4,6 +4,8 @@ last warp that is not full), idle lanes and bands, chains of their own warps,
 clusters with slabs of unequal height, both tile shapes, a source, the
 WaveHoltz tolerance, rank-local rectangles, non-square elements.
 
+The same for the one-element-per-thread kernel on curved quadrilaterals.
+
 Bounds: FP64 1e-12 and FP32 fp32_bound (the bounds of the other kernels: the
 tiles sum the same terms in another order); the tolerance mode may stop one
 iteration apart near the threshold, so it is bounded by 10 x the tolerance.
@@ -89,3 +91,35 @@ def test_tile_rectangles_equal_the_whole_sweep_bitwise(hz, monkeypatch, sx, sy, 
     assert np.array_equal(_host_c(u).reshape(whole_u.shape), whole_u)
     assert np.array_equal(_host_c(lout).reshape(whole_l.shape), whole_l)
     case.close()
+
+
+@pytest.mark.parametrize("nx,ny,sx,sy,P", [
+    (3, 3, 1, 1, 2),      # one element, 32 subdomains per warp
+    (12, 4, 4, 4, 3),     # 3 subdomains, 2 per warp
+    (16, 16, 8, 8, 3),    # the curved benchmark's subdomain: 2 warps
+    (10, 12, 5, 6, 4),    # idle lanes
+    (34, 6, 17, 3, 1),    # 17 of 32 lanes
+])
+def test_curved_tile_sweep_matches_oracle(hz, monkeypatch, nx, ny, sx, sy, P):
+    from paper_2606_21695_gb300.api import Case
+    from oracle import geom, sem
+    from workloads import configs
+
+    monkeypatch.setenv("HZ_SWEEP_VARIANT", "tile")
+    for robin in ((0.0, 1.0), (0.3, 0.8)):
+        wl = configs.Workload("ct", (0.0, 1.0, 0.0, 0.8), nx, ny, P, sx, sy, 9.0, "channel", (0.37, 0.48), 0.08,
+                              extra={"warp": 0.04})
+        case = Case(wl)
+        hz.hz_problem_set(case.pr, hz.HZ_TRANSMISSION, np.array(robin))
+        m = sem.Mesh(*wl.box, nx, ny, P, sx, sy)
+        X, Y = wl.node_xy(*m.coords_1d())
+        pr = geom.MappedProblem(m, X, Y, wl.speed_at(X, Y), wl.omega, wl.source_at(X, Y), wl.boundary(), robin=robin)
+        nt, lam = hz.hz_problem_nt(case.pr), _rand_lam(pr, 8)
+        for with_rhs in (True, False):
+            got_l, got_u = _run_sweep(hz, case, pr, hz.HZ_FP32_REFINE, nt, 3, lam, with_rhs)
+            ref_l, ref_u, _ = pr.sweep(lam, pr.rhs() if with_rhs else None, nt, 3, want_u=True)
+            assert _rel(got_u, ref_u) < _tol.FP32_REL and _rel(got_l, ref_l) < _tol.FP32_REL, (robin, with_rhs)
+        _, u = _run_sweep(hz, case, pr, hz.HZ_FP32_REFINE, nt, 30, lam, False, wh_tol=1e-3)
+        _, ref_u, _ = pr.sweep(lam, None, nt, 30, wh_tol=1e-3, want_u=True)
+        assert _rel(u, ref_u) < 1e-2
+        case.close()
