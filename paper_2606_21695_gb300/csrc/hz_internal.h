@@ -149,7 +149,7 @@ hz_status launch_sweep_cluster_f64(int P, const SweepArgs& a, int L, cudaStream_
 hz_status launch_sweep_cband(int P, const SweepArgs& a, int L, cudaStream_t st);
 
 // Sweep by element tiles (hz_sweep_tile.cuh): subdomains of at most 32 x 32
-// elements, degree 1..5 (FP64: 1..4, with a source 1..3), eta = 0, cold start.
+// elements, degree 1..5 (FP64: 1..4), eta = 0, cold start.
 // a.ty_force: 1 = one element per tile, 2 = two, paired (FP32, P <= 4, even
 // sub_ny), 0 = by size (tile_shape).  *warps: warps per subdomain, 0 for a
 // cluster.  HZ_ERR_UNSUPPORTED (nothing launched) else.
@@ -160,11 +160,11 @@ int tile_shape(bool fp32, int P, int sxe, int sye, int L);
 bool tile_default(bool fp32, int P, int sxe, int sye, int L);
 // Largest block of a tile shape.  Registers are allocated per scheduler (a
 // quarter of the SM's 65536), so a thread has 255 of them in blocks of up to
-// 8 warps, 168 up to 12, 128 up to 16, 80 up to 24.  A tile needs 5 (with a
-// source 7) values per node and 50 to 80 registers more for coefficients,
-// addresses and temporaries.
-constexpr int tile_max_threads(bool f64, int P, int H, bool src) {
-  const int words = P * P * H * (src ? 7 : 5) * (f64 ? 2 : 1);
+// 8 warps, 168 up to 12, 128 up to 16, 80 up to 24.  A tile needs 5 values
+// per node and 50 to 80 registers more for coefficients, addresses and
+// temporaries.
+constexpr int tile_max_threads(bool f64, int P, int H) {
+  const int words = P * P * H * 5 * (f64 ? 2 : 1);
   return words <= 10 ? 768 : words <= 40 ? 512 : words <= 90 ? 384 : 256;
 }
 constexpr int tile_pow2(int n) {  // smallest power of two >= n

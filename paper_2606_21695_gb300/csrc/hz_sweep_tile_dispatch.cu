@@ -37,7 +37,7 @@ int tile_shape(bool fp32, int P, int sxe, int sye, int L) {
   if (lanes1 <= 32 && sxe + sye <= 32) return 1;  // one warp either way
   if (lanes2 > 32 && (P == 4 || lanes2 % 32)) return 1;
   if (P == 1) return 2;
-  const int cap = tile_max_threads(false, P, 1, false) / 32;
+  const int cap = tile_max_threads(false, P, 1) / 32;
   const int warps = (lanes1 + 31) / 32 + (sxe + sye + 31) / 32;
   const int ctas = (warps + cap - 1) / cap;                     // CTAs per subdomain
   const int res = cap / ((warps + ctas - 1) / ctas);            // and per SM

@@ -29,7 +29,7 @@ hz_status launch_tile_iso(const SweepArgs& a0, int count, cudaStream_t st, int* 
     x.gs = tile_pow2(need);
     x.spw = 32 / x.gs;
     x.offB = sye;
-    const Lay y = make_lay<P, Real>(H, x.LX, x.nb, x.gs, tol);
+    const Lay y = make_lay<P, Real>(H, x.LX, x.nb, x.gs, SRC, tol);
     const size_t smem = (size_t)x.spw * y.total * sizeof(Real);
     auto kern = sweep_tile_kernel<Real, P, H, true, SRC, ISO, 32>;
     if (smem > 48 * 1024) HZ_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
@@ -39,7 +39,7 @@ hz_status launch_tile_iso(const SweepArgs& a0, int count, cudaStream_t st, int* 
     *warps = 1;
     return HZ_OK;
   }
-  constexpr int MAXT = tile_max_threads(sizeof(Real) == 8, P, H, SRC);
+  constexpr int MAXT = tile_max_threads(sizeof(Real) == 8, P, H);
   for (int CL = 1; CL <= 8; ++CL) {
     x.nb = (x.nbt + CL - 1) / CL;
     if (x.nbt - (CL - 1) * x.nb < 1) break;
@@ -48,7 +48,7 @@ hz_status launch_tile_iso(const SweepArgs& a0, int count, cudaStream_t st, int* 
     x.offB = nA + sxe <= 32 ? nA : 32;
     const int threads = 32 * (x.wm + (x.offB + sxe + 31) / 32);
     if (threads > MAXT) continue;
-    const Lay y = make_lay<P, Real>(H, x.LX, x.nb, threads, tol);
+    const Lay y = make_lay<P, Real>(H, x.LX, x.nb, threads, SRC, tol);
     const size_t smem = (size_t)y.total * sizeof(Real);
     if (smem > 220 * 1024) continue;
     auto kern = sweep_tile_kernel<Real, P, H, false, SRC, ISO, MAXT>;
@@ -79,29 +79,20 @@ hz_status launch_tile(const SweepArgs& a, int count, cudaStream_t st, int* warps
   return launch_tile_iso<Real, P, H, SRC, false>(a, count, st, warps);
 }
 
-// FP32, shape 1: one element per tile, shape 2: two, paired (P <= 4, with a
-// source P <= 3: the state of two larger elements exceeds a thread's registers).
+// FP32, shape 1: one element per tile, shape 2: two, paired (P <= 4: the state
+// of two larger elements exceeds a thread's registers).
 template <int P>
 hz_status launch_tile_f32(int shape, const SweepArgs& a, int count, cudaStream_t st, int* warps) {
-  if (a.rhs) {
-    if constexpr (P <= 3) {
-      if (shape == 2) return launch_tile<float, P, 2, true>(a, count, st, warps);
-    }
-    return launch_tile<float, P, 1, true>(a, count, st, warps);
-  }
   if constexpr (P <= 4) {
-    if (shape == 2) return launch_tile<float, P, 2, false>(a, count, st, warps);
+    if (shape == 2)
+      return a.rhs ? launch_tile<float, P, 2, true>(a, count, st, warps) : launch_tile<float, P, 2, false>(a, count, st, warps);
   }
-  return launch_tile<float, P, 1, false>(a, count, st, warps);
+  return a.rhs ? launch_tile<float, P, 1, true>(a, count, st, warps) : launch_tile<float, P, 1, false>(a, count, st, warps);
 }
 
 template <int P>
 hz_status launch_tile_f64(const SweepArgs& a, int count, cudaStream_t st, int* warps) {
-  if (a.rhs) {
-    if constexpr (P <= 3) return launch_tile<double, P, 1, true>(a, count, st, warps);
-    return HZ_ERR_UNSUPPORTED;
-  }
-  return launch_tile<double, P, 1, false>(a, count, st, warps);
+  return a.rhs ? launch_tile<double, P, 1, true>(a, count, st, warps) : launch_tile<double, P, 1, false>(a, count, st, warps);
 }
 
 }  // namespace tile_sweep
