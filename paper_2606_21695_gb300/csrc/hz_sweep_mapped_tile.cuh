@@ -22,6 +22,7 @@
 #include <cuda_runtime.h>
 
 #include "hz_internal.h"
+#include "hz_norm_acc.cuh"
 
 namespace hz {
 namespace mapped_tile {
@@ -318,19 +319,24 @@ __global__ void __launch_bounds__(ONE ? 32 : 256) sweep_mapped_tile_kernel(const
       // per-subdomain stop; a shared node counts once, for the element it starts
       const float* st = sm + y.stash;
       double dn = 0.0, un = 0.0;
+      NormAcc acc;
+      float big = 0.f;
+#pragma unroll
+      for (int k = 0; k < N2; ++k) big = fmaxf(big, fmaxf(fabsf(v[k / M][k % M].x), fabsf(v[k / M][k % M].y)));
+      acc.start(big);
 #pragma unroll
       for (int b = 0; b < M; ++b)
 #pragma unroll
         for (int c = 0; c < M; ++c) {
           const int k = b * M + c;
           const float orr = st[(2 * k) * nthr + t], oi = st[(2 * k + 1) * nthr + t];
-          if (done) v[b][c] = make_float2(orr, oi);
           if (live && (c < P || lastx) && (b < P || lasty)) {
-            const double dr = (double)v[b][c].x - (double)orr, di = (double)v[b][c].y - (double)oi;
-            dn += dr * dr + di * di;
-            un += (double)v[b][c].x * v[b][c].x + (double)v[b][c].y * v[b][c].y;
+            acc.add(v[b][c].x, orr);
+            acc.add(v[b][c].y, oi);
           }
+          if (done) v[b][c] = make_float2(orr, oi);
         }
+      acc.finish(dn, un);
       if (ONE) {
         for (int o = x.gs >> 1; o > 0; o >>= 1) {
           dn += __shfl_xor_sync(0xffffffffu, dn, o);

@@ -50,6 +50,7 @@
 
 #include "hz_gll_const.h"
 #include "hz_internal.h"
+#include "hz_norm_acc.cuh"
 
 namespace hz {
 namespace tile_sweep {
@@ -873,11 +874,33 @@ __device__ __forceinline__ void tile_body(const TileArgs& x, unsigned char* smem
       // group of a shared warp that has stopped keeps its iterate.
       const Real* st = sm + y.stash;
       double dn = 0.0, un = 0.0;
+      NormAcc acc;
+      if constexpr (sizeof(Real) == 4) {
+        float big = 0.f;
+        if (live) {
+#pragma unroll
+          for (int r = 0; r < P; ++r)
+#pragma unroll
+            for (int c = 0; c < P; ++c)
+#pragma unroll
+              for (int h = 0; h < H; ++h)
+                big = fmaxf(big, fmaxf(fabsf(get<H>(v[r][c].a, h)), fabsf(get<H>(v[r][c].b, h))));
+        }
+#pragma unroll
+        for (int q = 0; q <= P; ++q)
+          if (q < P ? inE : corner) big = fmaxf(big, fmaxf(fabsf(ev[q].a), fabsf(ev[q].b)));
+        acc.start(big);
+      }
       int k = 0;
       auto count = [&](Real nr, Real ni, Real orr, Real oi) {
-        const double dr = (double)nr - (double)orr, di = (double)ni - (double)oi;
-        dn += dr * dr + di * di;
-        un += (double)nr * nr + (double)ni * ni;
+        if constexpr (sizeof(Real) == 4) {
+          acc.add(nr, orr);
+          acc.add(ni, oi);
+        } else {
+          const double dr = nr - orr, di = ni - oi;
+          dn += dr * dr + di * di;
+          un += nr * nr + ni * ni;
+        }
       };
 #pragma unroll
       for (int r = 0; r < P; ++r)
@@ -886,21 +909,22 @@ __device__ __forceinline__ void tile_body(const TileArgs& x, unsigned char* smem
 #pragma unroll
           for (int h = 0; h < H; ++h, ++k) {
             const Real orr = st[(2 * k) * nthr + t], oi = st[(2 * k + 1) * nthr + t];
+            if (live) count(get<H>(v[r][c].a, h), get<H>(v[r][c].b, h), orr, oi);
             if (done) {
               put_half<H>(v[r][c].a, h, orr);
               put_half<H>(v[r][c].b, h, oi);
             }
-            if (live) count(get<H>(v[r][c].a, h), get<H>(v[r][c].b, h), orr, oi);
           }
 #pragma unroll
       for (int q = 0; q <= P; ++q, ++k) {
         const Real orr = st[(2 * k) * nthr + t], oi = st[(2 * k + 1) * nthr + t];
+        if (q < P ? inE : corner) count(ev[q].a, ev[q].b, orr, oi);
         if (done) {
           ev[q].a = orr;
           ev[q].b = oi;
         }
-        if (q < P ? inE : corner) count(ev[q].a, ev[q].b, orr, oi);
       }
+      if constexpr (sizeof(Real) == 4) acc.finish(dn, un);
       if (FUSE) {
         for (int o = x.gs >> 1; o > 0; o >>= 1) {
           dn += __shfl_xor_sync(0xffffffffu, dn, o);
