@@ -803,14 +803,14 @@ def run_ours(args):
             "peaks": peaks,
             "fp64_solve": fp64,
             "solve": {"sweeps_per_solve": sweeps / args.steps, "rel_residual_max": max(res),
-                      "sweep_kernel": {1: "block", 2: "warp", 3: "cluster", 4: "packed",
-                                       5: "cluster of warp bands", 6: "mapped (element form)"}.get(reports[0]["sweep_variant"]),
+                      "sweep_kernel": {1: "block", 2: "warps (element tiles or node columns)", 3: "cluster", 4: "packed",
+                                       5: "cluster of warps", 6: "mapped (element form)"}.get(reports[0]["sweep_variant"]),
                       "refinements": reports[0]["refinements"], "gmres_iters": reports[0]["gmres_iters"],
                       "dof_updates_per_solve": dof / args.steps},
             "roofline": {"kernel": {1: "sweep_kernel (block)",
-                                    2: ("sweep_warp_kernel (one warp per subdomain)" if reports[0]["sweep_shape"] <= 1
-                                        else f"sweep_band_kernel ({reports[0]['sweep_shape']} warps per subdomain)"),
-                                    3: "sweep_cluster_kernel", 5: "sweep_cband_kernel",
+                                    2: ("sweep_tile_kernel (element tiles) or a node-column kernel, "
+                                        f"{max(reports[0]['sweep_shape'], 1)} warp(s) per subdomain"),
+                                    3: "sweep_cluster_kernel", 5: "sweep_tile_kernel or sweep_cband_kernel on clusters",
                                     6: "sweep_mapped_kernel (element form, block per subdomain)"}.get(reports[0]["sweep_variant"], "?")
                          + " FP32, one launch = one DD sweep", "bound": "alu",
                          "achieved": achieved, "peak": peaks["fp32_tflops"], "unit": "TFLOP/s",

@@ -15,8 +15,8 @@
  *     point equal to the global discrete solution)
  *   - each subdomain solved by WaveHoltz (Sec. 5, eq. (WaveHoltz), modified
  *     leapfrog), all subdomains in one launch per DD sweep (Sec. 6,
- *     Algorithm 1): one warp, a few warps, one block or one thread-block
- *     cluster per subdomain, by subdomain size
+ *     Algorithm 1): part of a warp, one warp, a few warps, one block or one
+ *     thread-block cluster per subdomain, by subdomain size
  *   - outer iteration: GMRES on the transmission data (Sec. 3, Krylov
  *     acceleration) inside FP64 refinement on the global residual, defect
  *     correction or flexible GMRES (Sec. 7: the DD cycle is a preconditioner
@@ -172,8 +172,9 @@ typedef struct {
   double seconds;        /* wall time of the solve */
   int64_t dof_updates;   /* sum over sweeps of subdomain nodes x (N_t - 1) x WaveHoltz iterations */
   int32_t gmres_iters;   /* total GMRES iterations */
-  int32_t sweep_variant; /* kernel of the last sweep: 1 block, 2 warp per subdomain, 3 cluster,
-                            4 packed with other solves, 5 cluster of warp bands, 6 mapped mesh */
+  int32_t sweep_variant; /* kernel of the last sweep: 1 block, 2 warps per subdomain (element tiles or
+                            node columns), 3 cluster, 4 packed with other solves, 5 cluster of warps
+                            (element tiles or bands), 6 mapped mesh */
   int32_t sweep_shape;   /* its configuration: warps per subdomain (2), rows per thread in units
                             of the degree (1, 3; 0 = chosen by size) */
   double sweep_seconds;  /* device time of the sweep kernels (CUDA events on the solve's stream) */

@@ -150,7 +150,7 @@ hz_status launch_sweep_cband(int P, const SweepArgs& a, int L, cudaStream_t st);
 
 // Sweep by element tiles (hz_sweep_tile.cuh): subdomains of at most 32 x 32
 // elements, degree 1..5 (FP64: 1..4), eta = 0, cold start.
-// a.ty_force: 1 = one element per tile, 2 = two, paired (FP32, P <= 4, even
+// a.ty_force: 1 = one element per tile, 2 = two, paired (FP32, P <= 3, even
 // sub_ny), 0 = by size (tile_shape).  *warps: warps per subdomain, 0 for a
 // cluster.  HZ_ERR_UNSUPPORTED (nothing launched) else.
 hz_status launch_sweep_tile(bool fp32, int P, const SweepArgs& a, int count, cudaStream_t st, int* warps);

@@ -214,9 +214,8 @@ hz_status ensure_flags(Problem& pr) {
   return HZ_OK;
 }
 
-// Sweep kernel selection: HZ_SWEEP_VARIANT=block|warp|cluster forces one (tests);
-// default: the warp-per-subdomain kernel when compiled for the shape, else
-// the block kernel.
+// Sweep kernel selection: HZ_SWEEP_VARIANT=tile|block|warp|cluster|cband forces
+// one (tests); default: see sweep().
 int sweep_variant() {
   const char* v = std::getenv("HZ_SWEEP_VARIANT");
   if (!v) return kVariantAuto;
@@ -363,9 +362,9 @@ namespace {
 std::mutex g_tune_run_mu;
 }
 
-// Autotuner: times every sweep kernel variant that supports the shape (warp
-// per subdomain; one block per subdomain with P or 2P rows per thread; a
-// cluster of blocks) on this problem and caches the fastest per shape key.
+// Autotuner: times every sweep kernel variant that supports the shape (element
+// tiles of one or two elements; warp per subdomain; one block per subdomain
+// with P or 2P rows per thread; a cluster of blocks) on this problem and caches the fastest per shape key.
 hz_status autotune(Problem& pr, int precision, int nt, int m_wh, cudaStream_t st) {
   const std::string key = tune_key(pr.g, precision);
   Choice c{};
@@ -497,11 +496,12 @@ hz_status sweep(Problem& pr, int precision, int nt, int m_wh, double wh_tol, con
     }
   }
   // Kernel choice: HZ_SWEEP_VARIANT forces a variant; otherwise the tuned
-  // choice for this shape (if autotuning ran) or the size heuristic:
-  // FP32 -> warp-per-subdomain kernel when compiled for the shape, else one
-  // block per subdomain when it fits in 256 threads, else a cluster of
-  // blocks, else the block kernel with up to 1024 threads; FP64 -> block,
-  // else (subdomains too large for one block) a cluster of blocks.
+  // choice for this shape (if autotuning ran) or the size heuristic: the
+  // element tiles where tile_default says so; else FP32 -> warp-per-subdomain
+  // kernel when compiled for the shape, else one block per subdomain when it
+  // fits in 256 threads, else a cluster of blocks, else the block kernel with
+  // up to 1024 threads; FP64 -> block, else (subdomains too large for one
+  // block) a cluster of blocks.
   // a warm start (u0) is read by the one-warp and block kernels (and the
   // mapped kernel above); route it to those
   if (u0) {

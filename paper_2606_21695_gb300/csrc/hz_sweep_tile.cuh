@@ -29,16 +29,19 @@
 // share a warp), which also runs the chains; the barrier is __syncwarp.
 // Otherwise the chains have warps of their own, and subdomains whose state
 // exceeds one SM's registers take a thread-block cluster, each CTA a slab of
-// bands (exchange across slabs through distributed shared memory).
+// bands, whose end warps exchange with the neighbouring slabs' through
+// distributed shared memory (st.async with mbarriers).
 //
 // Bound: the FMA pipe at 19 FMAs per node and step (P = 3); what keeps it from
 // there is the chains (a sixth of a fused warp's instructions, on half of its
-// lanes), 1.7 warps per scheduler at 1024 one-warp subdomains, and on clusters
-// the barrier per step.  Measured, 20 WaveHoltz iterations: 1024 subdomains of
-// 25 x 25 nodes, P = 3, N_t = 55: 1073 us with the one-warp column kernel
-// (hz_sweep_warp.cuh: 4 shuffles and 30 instructions per node row and step),
-// 667 us here; 1024 of 129 x 129 nodes, P = 4, N_t = 48: 59.8 ms with the
-// cluster of warp bands, 108.6 ms with the cluster kernel, 25.5 ms here.
+// lanes) and the few warps that the registers leave room for (1.7 per
+// scheduler at 1024 one-warp subdomains).  Measured, 20 WaveHoltz iterations:
+// 1024 subdomains of 25 x 25 nodes, P = 3, N_t = 55: 1073 us with the one-warp
+// column kernel (hz_sweep_warp.cuh: 4 shuffles and 30 instructions per node row
+// and step), 602 us here; 16 of 17 x 17, P = 2, N_t = 79: 610, 168 us; 1024 of
+// 129 x 129, P = 4, N_t = 48: 59.8 ms with the cluster of warp bands, 108.6 ms
+// with the cluster kernel, 22.4 ms here.  A launch with clusters is a separate
+// instantiation: its few branches per step alone cost the others 20 to 40%.
 //
 // Taken by size (tile_shape, tile_default in hz_sweep_tile_dispatch.cu):
 // sxe <= 32 and sye <= 32 elements, fixed WaveHoltz count or per-subdomain
@@ -276,6 +279,26 @@ struct RowBuf<P, float> {
     if (kP1) v[4 * kQ < P ? 4 * kQ : 0] = buf[4 * kQ * n + idx];
   }
   static __device__ __forceinline__ float* first(float* buf, int idx) { return buf + (kQ ? 4 : kP2 ? 2 : 1) * idx; }
+  // the same store into another CTA's buffer, signalled to its mbarrier
+  static constexpr int kBytes = 16 * kQ + (kP2 ? 8 : kP1 ? 4 : 0);
+  static __device__ __forceinline__ void st_async(unsigned buf, int n, int idx, const float (&v)[P], unsigned mb) {
+#pragma unroll
+    for (int f = 0; f < kQ; ++f)
+      asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(
+                       buf + 16 * (f * n + idx)),
+                   "f"(at(v, 4 * f)), "f"(at(v, 4 * f + 1)), "f"(at(v, 4 * f + 2)), "f"(at(v, 4 * f + 3)), "r"(mb)
+                   : "memory");
+    if (kP2)
+      asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.f32 [%0], {%1, %2}, [%3];" ::"r"(
+                       buf + 16 * kQ * n + 8 * idx),
+                   "f"(at(v, 4 * kQ)), "f"(at(v, 4 * kQ + 1)), "r"(mb)
+                   : "memory");
+    if (kP1) st_async1(buf + 16 * kQ * n + 4 * idx, at(v, 4 * kQ), mb);
+  }
+  static __device__ __forceinline__ void st_async1(unsigned addr, float v, unsigned mb) {
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.f32 [%0], %1, [%2];" ::"r"(addr), "f"(v), "r"(mb)
+                 : "memory");
+  }
 };
 template <int P>
 struct RowBuf<P, double> {
@@ -296,6 +319,20 @@ struct RowBuf<P, double> {
     if (P % 2) v[P - 1] = buf[2 * kD * n + idx];
   }
   static __device__ __forceinline__ double* first(double* buf, int idx) { return buf + (kD ? 2 : 1) * idx; }
+  static constexpr int kBytes = 8 * P;
+  static __device__ __forceinline__ void st_async(unsigned buf, int n, int idx, const double (&v)[P], unsigned mb) {
+#pragma unroll
+    for (int f = 0; f < kD; ++f)
+      asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.f64 [%0], {%1, %2}, [%3];" ::"r"(
+                       buf + 16 * (f * n + idx)),
+                   "d"(v[2 * f]), "d"(v[2 * f + 1]), "r"(mb)
+                   : "memory");
+    if (P % 2) st_async1(buf + 16 * kD * n + 8 * idx, v[P - 1], mb);
+  }
+  static __device__ __forceinline__ void st_async1(unsigned addr, double v, unsigned mb) {
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.f64 [%0], %1, [%2];" ::"r"(addr), "d"(v), "r"(mb)
+                 : "memory");
+  }
 };
 
 // p and p-dot of a node, and its two filter sums: for FP32 scalars each pair
@@ -376,21 +413,57 @@ struct TileArgs {
 // registers; they meet at the same barriers.
 enum Role { kBoth = 0, kTiles = 1, kChains = 2 };
 
-struct TolShared {  // tolerance mode: per-warp and per-CTA partial norms, the decision
+struct TolShared {
+  unsigned long long mbar[2][4];  // clusters: arrivals by step parity
+  // tolerance mode: per-warp and per-CTA partial norms, the decision
   double red[32][2];
   double part[2];
   int stop;
 };
 
-// Cluster barrier in two halves: what a thread wrote before the arrival is
-// seen by the cluster after the wait; work in between hides the latency.
-__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
-__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
+// ---- exchange between the slabs of a cluster.  A cluster barrier per step
+// costs every warp a release fence and the wait for the slowest CTA; here only
+// the warps at a slab's ends wait, for the bytes that the neighbouring slab
+// stores straight into their buffers (st.async counts them on an mbarrier):
+// 144 subdomains of 129 x 129 nodes, P = 4: 754 us with a cluster barrier per
+// step (arrival and wait apart), 652 us; 9 of 97 x 97, P = 3: 140, 103 us.
+// Barriers by step parity and by what arrives: a row of T (from the slab
+// before), a row of p (from the one after), chain A's T and p.
+enum { kTilePrev = 0, kTileNext = 1, kChainPrev = 2, kChainNext = 3 };
+__device__ __forceinline__ unsigned smem_addr(const void* q) { return (unsigned)__cvta_generic_to_shared(q); }
+__device__ __forceinline__ unsigned peer_addr(unsigned addr, int rank) {
+  unsigned r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ void mbar_init(unsigned mb) { asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(mb) : "memory"); }
+__device__ __forceinline__ void mbar_expect(bool on, unsigned mb, unsigned bytes) {
+  asm volatile(
+      "{ .reg .pred q; .reg .b64 t; setp.ne.u32 q, %0, 0; @q mbarrier.arrive.expect_tx.shared::cta.b64 t, [%1], %2; }" ::"r"(
+          (unsigned)on),
+      "r"(mb), "r"(bytes)
+      : "memory");
+}
+// Waits for the phase; false after about a second (the caller records it and
+// stops waiting: a slab that never answers must not hang the device).
+__device__ __forceinline__ bool mbar_wait(unsigned mb, unsigned phase) {
+  const long long t0 = clock64();
+  do {
+    unsigned ok;
+    asm volatile(
+        "{ .reg .pred q; mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 q, [%1], %2; selp.u32 %0, 1, 0, q; }"
+        : "=r"(ok)
+        : "r"(mb), "r"(phase)
+        : "memory");
+    if (ok) return true;
+  } while (clock64() - t0 < 2000000000LL);
+  return false;
+}
 
 // Block barrier met by warps at different places of the program (the roles).
 __device__ __forceinline__ void block_bar() { asm volatile("bar.sync 0;" ::: "memory"); }
 
-template <typename Real, int P, int H, int ROLE, bool SRC, bool ISO>
+template <typename Real, int P, int H, int ROLE, bool SRC, bool ISO, bool CLUS>
 __device__ __forceinline__ void tile_body(const TileArgs& x, unsigned char* smem_raw, TolShared* ts) {
   constexpr bool FUSE = ROLE == kBoth, MAIN = ROLE != kChains, CHAIN = ROLE != kTiles;
   using V = typename VecT<Real, H>::V;
@@ -398,9 +471,9 @@ __device__ __forceinline__ void tile_body(const TileArgs& x, unsigned char* smem
   constexpr int RH = H * P;  // node rows of a tile
   const SweepArgs& a = x.base;
   cg::cluster_group cluster = cg::this_cluster();
-  const int CL = FUSE ? 1 : (int)cluster.num_blocks();
-  const int rk = FUSE ? 0 : (int)cluster.block_rank();
-  const bool firstC = rk == 0, lastC = rk == CL - 1;
+  const int CL = CLUS ? (int)cluster.num_blocks() : 1;
+  const int rk = CLUS ? (int)cluster.block_rank() : 0;
+  const bool firstC = !CLUS || rk == 0, lastC = !CLUS || rk == CL - 1;
   const int LX = x.LX;
   const int lane = threadIdx.x & 31;
   const int grp = FUSE ? lane / x.gs : 0;
@@ -429,11 +502,6 @@ __device__ __forceinline__ void tile_body(const TileArgs& x, unsigned char* smem
   const Lay y = make_lay<P, Real>(H, LX, x.nb, nthr, SRC, a.wh_tol > 0.0);
   const int ncol = x.nb * H + 1;  // elements of a column buffer
   Real* sm = reinterpret_cast<Real*>(smem_raw) + (FUSE ? grp * y.total : 0);
-  // slabs of a cluster: the previous CTA takes this slab's first row, the
-  // next one the T of its last band and chain A element
-  Real* smPrev = (!FUSE && !firstC) ? cluster.map_shared_rank(sm, rk - 1) : nullptr;
-  Real* smNext = (!FUSE && !lastC) ? cluster.map_shared_rank(sm, rk + 1) : nullptr;
-
   const int64_t nn = (int64_t)nlx * nly;
   const Real* betaG = static_cast<const Real*>(a.beta) + (int64_t)l * nn;
   const Real* alphaG = static_cast<const Real*>(a.alpha) + (int64_t)l * nn;
@@ -536,7 +604,23 @@ __device__ __forceinline__ void tile_body(const TileArgs& x, unsigned char* smem
       ebi[q] = (Real)(be * bi);
     }
   }
-  if (!FUSE && CL > 1) cluster.sync();  // every CTA of the cluster runs before its shared memory is written
+  unsigned mb0 = 0, mbP = 0, mbN = 0, smP = 0, smN = 0;  // this slab's barriers; the neighbours' barriers and buffers
+  if constexpr (CLUS) {
+    mb0 = smem_addr(ts->mbar);
+    if (threadIdx.x == 0) {
+      for (int k = 0; k < 8; ++k) mbar_init(mb0 + 8 * k);
+      asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (!firstC) {
+      mbP = peer_addr(mb0, rk - 1);
+      smP = peer_addr(smem_addr(sm), rk - 1);
+    }
+    if (!lastC) {
+      mbN = peer_addr(mb0, rk + 1);
+      smN = peer_addr(smem_addr(sm), rk + 1);
+    }
+  }
+  if (CLUS) cluster.sync();  // every CTA's buffers and barriers are ready before a neighbour uses them
   else if (FUSE) __syncwarp();
   else block_bar();
 
@@ -552,7 +636,17 @@ __device__ __forceinline__ void tile_body(const TileArgs& x, unsigned char* smem
   const Real rye = lo(ry), ryle = lo(ryl);
   const bool firstx = bx == 0, lastx = live && bx == sxe - 1;
   const bool firsty = by == 0 && firstC;
+  // slabs of a cluster: the slab before takes this one's first row, the next
+  // one the T of its last band; the warps that hold these bands wait for the
+  // neighbours' in turn, their first thread announces the bytes
   const bool sendPrev = live && by == 0 && !firstC, sendNext = live && by == nb - 1 && !lastC;
+  const int w0 = (int)(threadIdx.x & ~31u);  // the warp's first thread: its bands are w0 / LX .. (w0 + 31) / LX
+  const bool waitPrev = MAIN && CLUS && !firstC && w0 == 0;
+  const bool waitNext = MAIN && CLUS && !lastC && w0 <= nb * LX - 1 && nb * LX - 1 <= w0 + 31;
+  const bool chainPrev = CHAIN && CLUS && !firstC && (int)(threadIdx.x >> 5) == x.wm;
+  const bool chainNext = CHAIN && CLUS && !lastC && (int)(threadIdx.x >> 5) == x.wm;
+  bool answered = true;
+  unsigned phase = 0;  // of the barriers of the current parity
   const bool tol = a.wh_tol > 0.0;
   // the tile's nodes on the west column and the south row: alpha - 1 and
   // beta b in registers (zero on the other tiles: no branch in the time loop)
@@ -672,9 +766,10 @@ __device__ __forceinline__ void tile_body(const TileArgs& x, unsigned char* smem
           RB::st(PY + by * y.row, LX, bx, p0);
           RB::st(TY + (by + 1) * y.row, LX, bx, th);
         }
-        if (!FUSE) {
-          if (sendPrev) RB::st(smPrev + y.py + cur * pr_ + x.nb * y.row, LX, bx, p0);
-          if (sendNext) RB::st(smNext + y.ty + cur * pr_, LX, bx, th);
+        if constexpr (CLUS) {
+          const unsigned z = sizeof(Real);
+          if (sendPrev) RB::st_async(smP + z * (y.py + cur * pr_ + x.nb * y.row), LX, bx, p0, mbP + 8 * (4 * cur + kTileNext));
+          if (sendNext) RB::st_async(smN + z * (y.ty + cur * pr_), LX, bx, th, mbN + 8 * (4 * cur + kTilePrev));
         }
         V Tx[P];
 #pragma unroll
@@ -710,12 +805,24 @@ __device__ __forceinline__ void tile_body(const TileArgs& x, unsigned char* smem
         if (inE) RB::st(inB ? PY + nb * y.row : CP, en, ei, tv);
         if (corner) *RB::first(CP, nA) = es[P].a;
         if (inB && lastE) *RB::first(TA, nA) = eT;
-        if (!FUSE) {
-          if (inA && e == 0 && !firstC) *RB::first(smPrev + y.cp + cur * y.col, ncol - 1) = es[0].a;
-          if (inA && lastE && !lastC) smNext[y.tax + cur] = eT;
+        if constexpr (CLUS) {
+          const unsigned z = sizeof(Real);
+          const int cpo = (int)(RB::first(sm + y.cp + cur * y.col, ncol - 1) - sm);
+          if (inA && e == 0 && !firstC) RB::st_async1(smP + z * cpo, es[0].a, mbP + 8 * (4 * cur + kChainNext));
+          if (inA && lastE && !lastC) RB::st_async1(smN + z * (y.tax + cur), eT, mbN + 8 * (4 * cur + kChainPrev));
         }
       }
-      if (!FUSE && CL > 1) cluster_arrive();
+      if constexpr (CLUS) {  // what the neighbours will store in this step (predicated: no divergence here)
+        const unsigned mb = mb0 + 32 * cur;
+        if constexpr (MAIN) {
+          mbar_expect(waitPrev && lane == 0, mb + 8 * kTilePrev, sxe * RB::kBytes);
+          mbar_expect(waitNext && lane == 0, mb + 8 * kTileNext, sxe * RB::kBytes);
+        }
+        if constexpr (CHAIN) {
+          mbar_expect(chainPrev && lane == 0, mb + 8 * kChainPrev, sizeof(Real));
+          mbar_expect(chainNext && lane == 0, mb + 8 * kChainNext, sizeof(Real));
+        }
+      }
       const V ct = bc<V>((Real)tb.x), st = bc<V>((Real)tb.y), kz = bc<V>((Real)tb.z), kw = bc<V>((Real)tb.w);
       // ---- the part of the stiffness that the tile's own nodes give:
       // A = X + (hx/hy)^2 Y (ISO: square elements), row by row with the row's
@@ -781,9 +888,14 @@ __device__ __forceinline__ void tile_body(const TileArgs& x, unsigned char* smem
             }
         }
       }
-      if (FUSE) __syncwarp();
-      else if (CL > 1) cluster_wait();
-      else block_bar();
+      if (FUSE || CLUS) __syncwarp();  // (clusters: 2% faster with the warps reconverged before the barrier, blocks slower)
+      if (!FUSE) block_bar();
+      if constexpr (CLUS) {
+        const unsigned mb = mb0 + 32 * cur;
+        if (answered && (MAIN ? waitPrev : chainPrev)) answered = mbar_wait(mb + 8 * (MAIN ? kTilePrev : kChainPrev), phase);
+        if (answered && (MAIN ? waitNext : chainNext)) answered = mbar_wait(mb + 8 * (MAIN ? kTileNext : kChainNext), phase);
+        __syncwarp();
+      }
       // ---- what the neighbours sent, and the update
       if constexpr (MAIN) {
         Real ey[P], ty[P];
@@ -824,7 +936,7 @@ __device__ __forceinline__ void tile_body(const TileArgs& x, unsigned char* smem
         RB::ld(inB ? TY + nb * y.row : TA, en, ei, cr);
         const Real cpn = *RB::first(CP, nA), ca = *RB::first(TA, nA);
         if (lastE) eext = cpn;
-        if (!FUSE && inA && e == 0) erec = sm[y.tax + cur];
+        if (CLUS && inA && e == 0) erec = sm[y.tax + cur];
         const Real ec = (Real)tb.x, esn = (Real)tb.y;
 #pragma unroll
         for (int q = 0; q < P; ++q) {
@@ -853,6 +965,7 @@ __device__ __forceinline__ void tile_body(const TileArgs& x, unsigned char* smem
         accumulate(ev[P], (Real)tb.z, (Real)tb.w, es[P]);
       }
       tb = tn;
+      if (CLUS) phase ^= cur;  // the barriers' phase turns when parity 1 has been used
       cur ^= 1;
     }
     // u^{(m+1)} = (2/N_t) v
@@ -956,17 +1069,17 @@ __device__ __forceinline__ void tile_body(const TileArgs& x, unsigned char* smem
           part[0] = D;
           part[1] = U;
         }
-        if (CL > 1) cluster.sync();
+        if (CLUS) cluster.sync();
         if (threadIdx.x == 0) {
           double D = 0.0, U = 0.0;
           for (int r = 0; r < CL; ++r) {
-            const double* pr = CL > 1 ? cluster.map_shared_rank(part, r) : part;
+            const double* pr = CLUS ? cluster.map_shared_rank(part, r) : part;
             D += pr[0];
             U += pr[1];
           }
           ts->stop = (D <= a.wh_tol * a.wh_tol * U) ? 1 : 0;
         }
-        if (CL > 1) cluster.sync();  // remote reads of part done, stop visible to the CTA
+        if (CLUS) cluster.sync();  // remote reads of part done, stop visible to the CTA
         else block_bar();
         if (ts->stop) break;
       }
@@ -992,7 +1105,7 @@ __device__ __forceinline__ void tile_body(const TileArgs& x, unsigned char* smem
   for (int q = 0; q <= P; ++q)
     if (q < P ? inE : corner)
       out(inA ? nlx - 1 : eB * P + q, inA ? row0 + e * P + q : nly - 1, ev[q].a, ev[q].b);
-  if (bad) atomicOr(a.flags, 1);
+  if (bad || (CLUS && !answered)) atomicOr(a.flags, 1);  // a silent neighbour is reported as a failed solve
   if (t == 0 && have && firstC && a.wh_iter_max) {
     atomicMax(a.wh_iter_max, m_done);
     atomicAdd(a.wh_iter_sum, (unsigned long long)m_done);
@@ -1001,7 +1114,7 @@ __device__ __forceinline__ void tile_body(const TileArgs& x, unsigned char* smem
   // their last reads lie behind the barrier below), so that every thread
   // takes entries of the transmission update.  W, E: local rows; S, N: columns
   if (FUSE) __syncwarp();
-  else if (CL > 1) cluster.sync();  // the neighbours' last pushes have landed
+  else if (CLUS) cluster.sync();  // the neighbours' last pushes have landed
   else block_bar();
   const int rowsC = nb * RH + (lastC ? 1 : 0);  // node rows of this slab
   const int nrow = nb * RH + 1;
@@ -1074,15 +1187,15 @@ __device__ __forceinline__ void tile_body(const TileArgs& x, unsigned char* smem
   }
 }
 
-template <typename Real, int P, int H, bool FUSE, bool SRC, bool ISO, int MAXT>
+template <typename Real, int P, int H, bool FUSE, bool SRC, bool ISO, bool CLUS, int MAXT>
 __global__ void __launch_bounds__(MAXT) sweep_tile_kernel(const __grid_constant__ TileArgs x) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   if constexpr (FUSE) {
-    tile_body<Real, P, H, kBoth, SRC, ISO>(x, smem_raw, nullptr);
+    tile_body<Real, P, H, kBoth, SRC, ISO, CLUS>(x, smem_raw, nullptr);
   } else {
     __shared__ TolShared ts;
-    if ((int)(threadIdx.x >> 5) < x.wm) tile_body<Real, P, H, kTiles, SRC, ISO>(x, smem_raw, &ts);
-    else tile_body<Real, P, H, kChains, SRC, ISO>(x, smem_raw, &ts);
+    if ((int)(threadIdx.x >> 5) < x.wm) tile_body<Real, P, H, kTiles, SRC, ISO, CLUS>(x, smem_raw, &ts);
+    else tile_body<Real, P, H, kChains, SRC, ISO, CLUS>(x, smem_raw, &ts);
   }
 }
 

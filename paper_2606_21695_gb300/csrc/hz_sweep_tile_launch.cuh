@@ -31,7 +31,7 @@ hz_status launch_tile_iso(const SweepArgs& a0, int count, cudaStream_t st, int* 
     x.offB = sye;
     const Lay y = make_lay<P, Real>(H, x.LX, x.nb, x.gs, SRC, tol);
     const size_t smem = (size_t)x.spw * y.total * sizeof(Real);
-    auto kern = sweep_tile_kernel<Real, P, H, true, SRC, ISO, 32>;
+    auto kern = sweep_tile_kernel<Real, P, H, true, SRC, ISO, false, 32>;
     if (smem > 48 * 1024) HZ_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     kern<<<(count + x.spw - 1) / x.spw, 32, smem, st>>>(x);
     note_launch();
@@ -51,7 +51,8 @@ hz_status launch_tile_iso(const SweepArgs& a0, int count, cudaStream_t st, int* 
     const Lay y = make_lay<P, Real>(H, x.LX, x.nb, threads, SRC, tol);
     const size_t smem = (size_t)y.total * sizeof(Real);
     if (smem > 220 * 1024) continue;
-    auto kern = sweep_tile_kernel<Real, P, H, false, SRC, ISO, MAXT>;
+    auto kern = CL > 1 ? sweep_tile_kernel<Real, P, H, false, SRC, ISO, true, MAXT>
+                       : sweep_tile_kernel<Real, P, H, false, SRC, ISO, false, MAXT>;
     if (smem > 48 * 1024) HZ_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)(count * CL));
@@ -79,11 +80,12 @@ hz_status launch_tile(const SweepArgs& a, int count, cudaStream_t st, int* warps
   return launch_tile_iso<Real, P, H, SRC, false>(a, count, st, warps);
 }
 
-// FP32, shape 1: one element per tile, shape 2: two, paired (P <= 4: the state
-// of two larger elements exceeds a thread's registers).
+// FP32, shape 1: one element per tile, shape 2: two, paired (P <= 3: the state
+// of two larger elements leaves too few warps; P = 4, 8 x 8 elements at 1024
+// subdomains: 235 us one by one, 241 paired, 16 x 16 at 256: 239, 264).
 template <int P>
 hz_status launch_tile_f32(int shape, const SweepArgs& a, int count, cudaStream_t st, int* warps) {
-  if constexpr (P <= 4) {
+  if constexpr (P <= 3) {
     if (shape == 2)
       return a.rhs ? launch_tile<float, P, 2, true>(a, count, st, warps) : launch_tile<float, P, 2, false>(a, count, st, warps);
   }
