@@ -609,6 +609,17 @@ static MappedGlobalArgs mapped_args(const Problem& pr) {
   return a;
 }
 
+// The residual's block counter, zero between launches.  hz_problem_create makes
+// it; problems that the server builds from a snapshot get theirs at their
+// first residual.
+hz_status ensure_ticket(Problem& pr) {
+  if (pr.ticket.ptr) return HZ_OK;
+  HZ_TRY(pr.ticket.ensure(16));
+  HZ_CUDA(cudaMemset(pr.ticket.ptr, 0, 16));
+  HZ_UPLOADS_DONE();
+  return HZ_OK;
+}
+
 hz_status residual(Problem& pr, const double* b, const double* u, double* r, double* norms2_dev, cudaStream_t st) {
   HZ_TRY(check_ready(pr));
   if (pr.mapped) {
@@ -621,11 +632,7 @@ hz_status residual(Problem& pr, const double* b, const double* u, double* r, dou
   }
   const GlobalArgs a = global_args(pr);
   HZ_TRY(pr.part.ensure((size_t)residual_blocks(a) * 2 * sizeof(double)));
-  if (!pr.ticket.ptr) {
-    HZ_TRY(pr.ticket.ensure(16));
-    HZ_CUDA(cudaMemset(pr.ticket.ptr, 0, 16));
-    HZ_UPLOADS_DONE();
-  }
+  HZ_TRY(ensure_ticket(pr));
   return launch_residual(a, b, u, r, pr.part.as<double>(), static_cast<unsigned*>(pr.ticket.ptr), norms2_dev, st);
 }
 
@@ -1407,6 +1414,7 @@ hz_status hz_problem_create(hz_mesh mesh, int32_t device, hz_problem* out) {
       const size_t nbd = (size_t)(2 * g.NXg + 2 * g.NYg) * 2 * sizeof(double);
       HZ_TRY(pr->gb.ensure(nbd));
       HZ_CUDA(cudaMemset(pr->gb.ptr, 0, nbd));
+      HZ_TRY(ensure_ticket(*pr));  // here, so that a residual's launch can be captured
       HZ_UPLOADS_DONE();
       HZ_CUDA(cudaStreamCreateWithFlags(&pr->stream, cudaStreamNonBlocking));
       return HZ_OK;

@@ -443,9 +443,12 @@ hz_status launch_src(const MappedSweepArgs& m, int count, cudaStream_t st) {
   x.gs = threads;
   x.spw = one ? 32 / threads : 1;
   const size_t smem = (size_t)x.spw * y.total * sizeof(float);
-  if (smem > 200 * 1024) return HZ_ERR_UNSUPPORTED;
+  // the kernel's limit is this constant and not the launch's own size: another
+  // thread's smaller launch would lower it between the two calls
+  constexpr int kMaxSmem = 200 * 1024;
+  if (smem > kMaxSmem) return HZ_ERR_UNSUPPORTED;
   auto kern = one ? sweep_mapped_tile_kernel<P, true, SRC> : sweep_mapped_tile_kernel<P, false, SRC>;
-  if (smem > 48 * 1024) HZ_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  if (smem > 48 * 1024) HZ_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem));
   kern<<<(count + x.spw - 1) / x.spw, one ? 32 : threads, smem, st>>>(x);
   note_launch();
   HZ_CUDA(cudaGetLastError());

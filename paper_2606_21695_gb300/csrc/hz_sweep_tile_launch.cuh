@@ -7,6 +7,11 @@
 namespace hz {
 namespace tile_sweep {
 
+// Dynamic shared memory that a launch may ask for.  A kernel's limit is set to
+// this constant and not to the launch's own size: another thread that launches
+// the same kernel with less would lower the limit between the two calls.
+constexpr int kMaxSmem = 220 * 1024;
+
 template <typename Real, int P, int H, bool SRC, bool ISO>
 hz_status launch_tile_iso(const SweepArgs& a0, int count, cudaStream_t st, int* warps) {
   const int sxe = a0.sxe, sye = a0.sye;
@@ -32,7 +37,7 @@ hz_status launch_tile_iso(const SweepArgs& a0, int count, cudaStream_t st, int* 
     const Lay y = make_lay<P, Real>(H, x.LX, x.nb, x.gs, SRC, tol);
     const size_t smem = (size_t)x.spw * y.total * sizeof(Real);
     auto kern = sweep_tile_kernel<Real, P, H, true, SRC, ISO, false, 32>;
-    if (smem > 48 * 1024) HZ_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    if (smem > 48 * 1024) HZ_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem));
     kern<<<(count + x.spw - 1) / x.spw, 32, smem, st>>>(x);
     note_launch();
     HZ_CUDA(cudaGetLastError());
@@ -50,10 +55,10 @@ hz_status launch_tile_iso(const SweepArgs& a0, int count, cudaStream_t st, int* 
     if (threads > MAXT) continue;
     const Lay y = make_lay<P, Real>(H, x.LX, x.nb, threads, SRC, tol);
     const size_t smem = (size_t)y.total * sizeof(Real);
-    if (smem > 220 * 1024) continue;
+    if (smem > kMaxSmem) continue;
     auto kern = CL > 1 ? sweep_tile_kernel<Real, P, H, false, SRC, ISO, true, MAXT>
                        : sweep_tile_kernel<Real, P, H, false, SRC, ISO, false, MAXT>;
-    if (smem > 48 * 1024) HZ_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    if (smem > 48 * 1024) HZ_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem));
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)(count * CL));
     cfg.blockDim = dim3((unsigned)threads);
