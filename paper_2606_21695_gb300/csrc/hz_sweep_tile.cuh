@@ -73,6 +73,10 @@ namespace cg = cooperative_groups;
 // those choices so that the second moments, weighted over the element's rows,
 // cancel (that is the relative error of the wave number, equal at every node)
 // with the first moments small.
+// FP64 rows are rounded one by one: against long double, 10 WaveHoltz iterations
+// on 25 x 25 nodes (P = 3, N_t = 55) are off by 1.7e-15 to 2e-15, by 4.3e-15 to
+// 5.6e-15 when Kref and the weights are applied one after the other, and by 3e-15
+// to 4e-15 with the diagonal as minus the sum.
 template <typename Real>
 struct TileRows {
   Real c[kMaxP][kMaxP + 1][kMaxP + 1] = {};
