@@ -38,7 +38,7 @@
 // scheduler at 1024 one-warp subdomains).  Measured, 20 WaveHoltz iterations:
 // 1024 subdomains of 25 x 25 nodes, P = 3, N_t = 55: 1073 us with the one-warp
 // column kernel (hz_sweep_warp.cuh: 4 shuffles and 30 instructions per node row
-// and step), 602 us here; 16 of 17 x 17, P = 2, N_t = 79: 610, 168 us; 1024 of
+// and step), 565 us here; 16 of 17 x 17, P = 2, N_t = 79: 610, 168 us; 1024 of
 // 129 x 129, P = 4, N_t = 48: 59.8 ms with the cluster of warp bands, 108.6 ms
 // with the cluster kernel, 22.4 ms here.  A launch with clusters is a separate
 // instantiation: its few branches per step alone cost the others 20 to 40%.
@@ -698,6 +698,11 @@ __device__ __forceinline__ void tile_body(const TileArgs& x, unsigned char* smem
 #pragma unroll
   for (int q = 0; q <= P; ++q) ev[q].a = ev[q].b = Real(0);
 
+  // Two steps per turn of the time loop, so that each parity's buffers are fixed
+  // offsets: 1024 subdomains of 25 x 25 nodes, P = 3: 602 us with one, 565 us.
+  // Not where it takes more registers than there are (P = 3 with a source: 52
+  // bytes spilled, P = 5: 96 to 256).
+  constexpr bool kTwo = FUSE && P <= 3 && !SRC;
   int cur = 0, m_done = 0;
   bool done = false;  // tolerance met (FUSE: this lane group; else the whole subdomain)
   for (int m = 0; m < a.m_wh; ++m) {
@@ -740,7 +745,10 @@ __device__ __forceinline__ void tile_body(const TileArgs& x, unsigned char* smem
       }
     }
     Tab tb = tab[1];
+    if (kTwo) __syncwarp();  // the first step may write the buffers that the last iteration's last step read
+#pragma unroll (kTwo ? 2 : 1)
     for (int nu = 1; nu < a.Nt; ++nu) {
+      if (kTwo) cur = nu & 1;
       const Tab tn = tab[nu + 1];  // prefetch (the table has N_t + 1 entries)
       Real* PY = sm + y.py + cur * pr_;
       Real* TY = sm + y.ty + cur * pr_;
@@ -970,7 +978,7 @@ __device__ __forceinline__ void tile_body(const TileArgs& x, unsigned char* smem
       }
       tb = tn;
       if (CLUS) phase ^= cur;  // the barriers' phase turns when parity 1 has been used
-      cur ^= 1;
+      if (!kTwo) cur ^= 1;
     }
     // u^{(m+1)} = (2/N_t) v
 #pragma unroll
