@@ -12,6 +12,7 @@
 
 #include <cmath>
 
+#include "hz_complex_io.cuh"
 #include "hz_internal.h"
 
 namespace hz {
@@ -153,28 +154,28 @@ struct ResNode {  // what a node adds to the two sums
   double rr = 0.0, bb = 0.0;
 };
 // S: the node's taps including its own value's
+template <bool PAIR>
 __device__ __forceinline__ void residual_node(int64_t n, double W, double h, double2 u, double2 S,
                                               const double* __restrict__ b, double* __restrict__ r, ResNode& sum) {
   double2 bn = make_double2(0.0, 0.0);
-  if (b) bn = reinterpret_cast<const double2*>(b)[n];
+  if (b) bn = load_complex<PAIR>(b, n);
   double rr = fma(-W, S.x, bn.x);
   double ri = fma(-W, S.y, bn.y);
   if (h != 0.0) {
     rr = fma(-h, u.y, rr);
     ri = fma(h, u.x, ri);
   }
-  reinterpret_cast<double2*>(r)[n] = make_double2(rr, ri);
+  store_complex<PAIR>(r, n, make_double2(rr, ri));
   sum.rr = fma(rr, rr, fma(ri, ri, sum.rr));
   if (b) sum.bb = fma(bn.x, bn.x, fma(bn.y, bn.y, sum.bb));
 }
 
-template <int P>
+template <int P, bool PAIR>
 __global__ void __launch_bounds__(32 * kResRows)
     residual_kernel(const __grid_constant__ GlobalArgs a, int nbx, int nmain, const double* __restrict__ b,
                     const double* __restrict__ u, double* __restrict__ r, double* __restrict__ part,
                     unsigned* __restrict__ ticket, double* __restrict__ norms2) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const double2* u2 = reinterpret_cast<const double2*>(u);
   ResNode sum;
   if ((int)blockIdx.x < nmain) {
     const int ex = (int)(blockIdx.x % nbx) * 32 + lane;
@@ -183,7 +184,7 @@ __global__ void __launch_bounds__(32 * kResRows)
       const int64_t n0 = (int64_t)J * a.NXg + (int64_t)ex * P;
       double2 v[P + 1], S[P];
 #pragma unroll
-      for (int k = 0; k <= P; ++k) v[k] = __ldg(&u2[n0 + k]);
+      for (int k = 0; k <= P; ++k) v[k] = load_complex_ro<PAIR>(u, n0 + k);
       // y: the element row's own nodes, and on a shared row the element below
       const int ay = J % P;
       const int cy = J == 0 ? P : J == a.NYg - 1 ? P + 1 : ay;
@@ -196,10 +197,10 @@ __global__ void __launch_bounds__(32 * kResRows)
       }
       auto yrow = [&](int off) {  // row J + off, 0 < |off| <= P
         const double cf = a.Ky[cy][P + off];
-        const double2* row = u2 + n0 + (int64_t)off * a.NXg;
+        const int64_t row = n0 + (int64_t)off * a.NXg;
 #pragma unroll
         for (int k = 0; k < P; ++k) {
-          const double2 w = __ldg(&row[k]);
+          const double2 w = load_complex_ro<PAIR>(u, row + k);
           S[k].x = fma(cf, w.x, S[k].x);
           S[k].y = fma(cf, w.y, S[k].y);
         }
@@ -223,7 +224,7 @@ __global__ void __launch_bounds__(32 * kResRows)
       if (ex > 0) {
 #pragma unroll
         for (int k = 1; k <= P; ++k) {
-          const double2 w = __ldg(&u2[n0 - k]);
+          const double2 w = load_complex_ro<PAIR>(u, n0 - k);
           S[0].x = fma(a.Kx[0][P - k], w.x, S[0].x);
           S[0].y = fma(a.Kx[0][P - k], w.y, S[0].y);
         }
@@ -243,7 +244,7 @@ __global__ void __launch_bounds__(32 * kResRows)
         const double Wx = a.Wxg[ex * P + q];
         double h = 0.0;
         if (yb || (q == 0 && ex == 0)) h = t[q] * ((yb ? Wx : 0.0) + (q == 0 && ex == 0 ? Wy : 0.0));
-        residual_node(n0 + q, Wx * Wy, h, v[q], S[q], b, r, sum);
+        residual_node<PAIR>(n0 + q, Wx * Wy, h, v[q], S[q], b, r, sum);
       }
     }
   } else {
@@ -253,23 +254,23 @@ __global__ void __launch_bounds__(32 * kResRows)
       const int64_t n = (int64_t)J * a.NXg + I;
       const int cy = J == 0 ? P : J == a.NYg - 1 ? P + 1 : J % P;
       const double t = a.omega * recip(a.c[n]), d = fma(-t, t, a.Kd[P + 1][cy]);
-      const double2 un = u2[n];
+      const double2 un = load_complex_ro<PAIR>(u, n);
       double2 S = make_double2(d * un.x, d * un.y);
       for (int k = -P; k <= P; ++k) {
         if (k == 0) continue;
         if (J + k >= 0 && J + k < a.NYg) {  // taps outside the row's class have coefficient 0
-          const double2 w = __ldg(&u2[n + (int64_t)k * a.NXg]);
+          const double2 w = load_complex_ro<PAIR>(u, n + (int64_t)k * a.NXg);
           S.x = fma(a.Ky[cy][P + k], w.x, S.x);
           S.y = fma(a.Ky[cy][P + k], w.y, S.y);
         }
         if (k < 0) {
-          const double2 w = __ldg(&u2[n + k]);
+          const double2 w = load_complex_ro<PAIR>(u, n + k);
           S.x = fma(a.Kx[P + 1][P + k], w.x, S.x);
           S.y = fma(a.Kx[P + 1][P + k], w.y, S.y);
         }
       }
       const double Wx = a.Wxg[I], Wy = a.Wyg[J];
-      residual_node(n, Wx * Wy, t * (Wy + (J == 0 || J == a.NYg - 1 ? Wx : 0.0)), un, S, b, r, sum);
+      residual_node<PAIR>(n, Wx * Wy, t * (Wy + (J == 0 || J == a.NYg - 1 ? Wx : 0.0)), un, S, b, r, sum);
     }
   }
   if (!norms2) return;
@@ -523,8 +524,11 @@ int residual_main_blocks(const GlobalArgs& a) { return (a.nx + 31) / 32 * ((a.NY
 template <int P>
 hz_status launch_residual_P(const GlobalArgs& a, const double* b, const double* u, double* r, double* part,
                             unsigned* ticket, double* norms2, cudaStream_t st) {
-  residual_kernel<P><<<residual_blocks(a), 32 * kResRows, 0, st>>>(a, (a.nx + 31) / 32, residual_main_blocks(a), b, u,
-                                                                   r, part, ticket, norms2);
+  // a caller's array off the 16-byte grid: entries as two doubles each
+  const bool pair = is_pair_aligned(b) && is_pair_aligned(u) && is_pair_aligned(r);
+  auto kern = pair ? residual_kernel<P, true> : residual_kernel<P, false>;
+  kern<<<residual_blocks(a), 32 * kResRows, 0, st>>>(a, (a.nx + 31) / 32, residual_main_blocks(a), b, u, r, part, ticket,
+                                                     norms2);
   note_launch();
   HZ_CUDA(cudaGetLastError());
   return HZ_OK;

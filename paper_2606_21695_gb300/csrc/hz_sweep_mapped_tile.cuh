@@ -21,6 +21,7 @@
 
 #include <cuda_runtime.h>
 
+#include "hz_complex_io.cuh"
 #include "hz_internal.h"
 #include "hz_norm_acc.cuh"
 
@@ -378,8 +379,8 @@ __global__ void __launch_bounds__(ONE ? 32 : 256) sweep_mapped_tile_kernel(const
       for (int c = 0; c < M; ++c) {
         if (!isfinite(v[b][c].x) || !isfinite(v[b][c].y)) bad = true;
         if (a.u_sub && (c < P || lastx) && (b < P || lasty))
-          reinterpret_cast<double2*>(a.u_sub)[(int64_t)l * nn + (int64_t)(ey * P + b) * nlx + ex * P + c] =
-              make_double2(v[b][c].x, v[b][c].y);
+          store_complex(a.u_sub, (int64_t)l * nn + (int64_t)(ey * P + b) * nlx + ex * P + c,
+                        make_double2(v[b][c].x, v[b][c].y));
       }
   }
   if (bad) atomicOr(a.flags, 1);
@@ -415,13 +416,13 @@ __global__ void __launch_bounds__(ONE ? 32 : 256) sweep_mapped_tile_kernel(const
           const float* us = sm + (ed == 0 ? y.tw : ed == 1 ? y.te : ed == 2 ? y.ts : y.tn) + 4 * q;
           const double ur = (double)us[0], ui = (double)us[1];
           const double kk = kedgeL[ed * NE + q];
-          const double2 lr = reinterpret_cast<const double2*>(lamL)[ed * NE + q];
+          const double2 lr = load_complex(lamL, ed * NE + q);
           // -lambda + 2 k (eta - i zeta) u
           w.x = -lr.x + 2.0 * kk * (a.eta * ur + a.zeta * ui);
           w.y = -lr.y + 2.0 * kk * (a.eta * ui - a.zeta * ur);
         }
       }
-      reinterpret_cast<double2*>(a.lam_out)[dst] = w;
+      store_complex(a.lam_out, dst, w);
     }
   }
 }

@@ -51,6 +51,7 @@
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
+#include "hz_complex_io.cuh"
 #include "hz_gll_const.h"
 #include "hz_internal.h"
 #include "hz_norm_acc.cuh"
@@ -521,7 +522,7 @@ __device__ __forceinline__ void tile_body(const TileArgs& x, unsigned char* smem
       const double shx = ((i == 0 && ifW) || (i == nlx - 1 && ifE)) ? 0.5 : 1.0;
       const double shy = ((j == 0 && ifS) || (j == nly - 1 && ifN)) ? 0.5 : 1.0;
       const int64_t I = (int64_t)sxi * a.snxP + i, J = (int64_t)syi * a.snyP + j;
-      const double2 s = reinterpret_cast<const double2*>(a.rhs)[J * a.NXg + I];
+      const double2 s = load_complex(a.rhs, J * a.NXg + I);
       br = shx * shy * s.x;
       bi = shx * shy * s.y;
     }
@@ -579,7 +580,7 @@ __device__ __forceinline__ void tile_body(const TileArgs& x, unsigned char* smem
           put_half<H>(nbet[r][c], h, (Real)(-be * wx * wy * sxs));
           if (SRC && i > 0 && j > 0) {  // first column and row: in the tables
             const int64_t I = (int64_t)sxi * a.snxP + i, J = (int64_t)syi * a.snyP + j;
-            const double2 s = reinterpret_cast<const double2*>(a.rhs)[J * a.NXg + I];
+            const double2 s = load_complex(a.rhs, J * a.NXg + I);
             put_half<H>(f.re, h, (Real)(be * s.x));
             put_half<H>(f.im, h, (Real)(be * s.y));
           }
@@ -1102,7 +1103,7 @@ __device__ __forceinline__ void tile_body(const TileArgs& x, unsigned char* smem
   bool bad = false;
   auto out = [&](int i, int j, Real re, Real im) {
     if (!isfinite(re) || !isfinite(im)) bad = true;
-    if (a.u_sub) reinterpret_cast<double2*>(a.u_sub)[(int64_t)l * nn + (int64_t)j * nlx + i] = make_double2(re, im);
+    if (a.u_sub) store_complex(a.u_sub, (int64_t)l * nn + (int64_t)j * nlx + i, make_double2(re, im));
   };
   if (live) {
 #pragma unroll
@@ -1188,13 +1189,13 @@ __device__ __forceinline__ void tile_body(const TileArgs& x, unsigned char* smem
           const Real* us = (ed == 0 ? uW : ed == 1 ? uE : ed == 2 ? uS : uN) + 2 * loc;
           const double ur = (double)us[0], ui = (double)us[1];
           const double kk = kedgeL[ed * NE + q];
-          const double2 lr = reinterpret_cast<const double2*>(lamL)[ed * NE + q];
+          const double2 lr = load_complex(lamL, ed * NE + q);
           // -lambda + 2 k (eta - i zeta) u, eta = 0
           v.x = -lr.x + 2.0 * kk * (a.eta * ur + a.zeta * ui);
           v.y = -lr.y + 2.0 * kk * (a.eta * ui - a.zeta * ur);
         }
       }
-      reinterpret_cast<double2*>(a.lam_out)[dst] = v;
+      store_complex(a.lam_out, dst, v);
     }
   }
 }
