@@ -34,9 +34,8 @@
  *     "stream" is a cudaStream_t (NULL = legacy default stream).  Device
  *     entry points enqueue work on that stream; they may synchronise it where
  *     noted.
- *   - Device arrays of hz_sweep, hz_sweep_from, hz_sweep_rect, hz_sweep_packed,
- *     hz_residual, hz_rhs and hz_assemble_add may start at any multiple of 8
- *     bytes (a complex entry need not be 16-byte aligned).
+ *   - Device arrays of doubles may start at any multiple of 8 bytes (a complex
+ *     entry need not be 16-byte aligned).
  *   - Calls on one problem handle are not thread-safe; server calls are.
  */
 #ifndef HZ_H

@@ -6,6 +6,7 @@
 // fluxes of u, one thread per global node for the assembly gather.
 #include <cuda_runtime.h>
 
+#include "hz_complex_io.cuh"
 #include "hz_internal.h"
 
 namespace hz {
@@ -40,7 +41,7 @@ __global__ void rhs_mapped_kernel(const __grid_constant__ MappedGlobalArgs a, co
 }
 
 // metric fluxes of u at every element node: flux[(e N2 + loc) 4 + {F1 re, F1 im, F2 re, F2 im}]
-template <int P>
+template <int P, bool PAIR>
 __global__ void flux_mapped_kernel(const __grid_constant__ MappedGlobalArgs a, const double* __restrict__ u) {
   constexpr int M = P + 1, N2 = M * M;
   const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -50,14 +51,13 @@ __global__ void flux_mapped_kernel(const __grid_constant__ MappedGlobalArgs a, c
   const int loc = (int)(idx - e * N2);
   const int b = loc / M, aa = loc - b * M;
   const int ex = (int)(e % a.nx), ey = (int)(e / a.nx);
-  const double2* u2 = reinterpret_cast<const double2*>(u);
   const int64_t row0 = ((int64_t)ey * P + b) * a.NXg + (int64_t)ex * P;
   const int64_t col0 = ((int64_t)ey * P) * a.NXg + (int64_t)ex * P + aa;
   double xr = 0, xi = 0, er = 0, ei = 0;
 #pragma unroll
   for (int c = 0; c < M; ++c) {
-    const double2 vr = u2[row0 + c];
-    const double2 vc = u2[col0 + (int64_t)c * a.NXg];
+    const double2 vr = load_complex<PAIR>(u, row0 + c);
+    const double2 vc = load_complex<PAIR>(u, col0 + (int64_t)c * a.NXg);
     xr += a.D[aa * M + c] * vr.x;
     xi += a.D[aa * M + c] * vr.y;
     er += a.D[b * M + c] * vc.x;
@@ -144,7 +144,8 @@ hz_status residual_mapped_P(const MappedGlobalArgs& a, const double* b, const do
                             int* nblocks, cudaStream_t st) {
   constexpr int N2 = (P + 1) * (P + 1);
   const int64_t total = (int64_t)a.nx * a.ny * N2;
-  flux_mapped_kernel<P><<<(unsigned)((total + 255) / 256), 256, 0, st>>>(a, u);
+  auto flux = is_pair_aligned(u) ? flux_mapped_kernel<P, true> : flux_mapped_kernel<P, false>;
+  flux<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(a, u);
   note_launch();
   HZ_CUDA(cudaGetLastError());
   dim3 blk(32, 8);

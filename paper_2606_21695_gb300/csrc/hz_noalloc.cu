@@ -21,6 +21,7 @@
 #include <mutex>
 #include <string>
 
+#include "hz_complex_io.cuh"
 #include "hz_internal.h"
 
 namespace hz {
@@ -71,7 +72,7 @@ __device__ __forceinline__ double warp_sum_na(double v) {
 // r = b - (A - i w H - w^2 M) u (Sec. 4), the lumped 1D weights formed on the
 // fly from the GLL weights (same products and summation order as the host
 // tables of hz_residual); per-block partial sums into the static scratch.
-template <int P>
+template <int P, bool PAIR>
 __global__ void residual_noalloc_kernel(const __grid_constant__ NoallocArgs a, const double* __restrict__ c,
                                         const double* __restrict__ b, const double* __restrict__ u,
                                         double* __restrict__ r, double* __restrict__ part) {
@@ -80,7 +81,6 @@ __global__ void residual_noalloc_kernel(const __grid_constant__ NoallocArgs a, c
   double s0 = 0.0, s1 = 0.0;
   if (I < a.NXg && J < a.NYg) {
     const int64_t n = (int64_t)J * a.NXg + I;
-    const double2* u2 = reinterpret_cast<const double2*>(u);
     const int ax = I % P, ex = I / P;
     const bool own_x = ex < a.nx, left_x = (ax == 0) && ex >= 1;
     double sxr = 0.0, sxi = 0.0;
@@ -92,7 +92,7 @@ __global__ void residual_noalloc_kernel(const __grid_constant__ NoallocArgs a, c
       if (in_own) cf += a.Kref[ax * (P + 1) + bb];
       if (in_left) cf += a.Kref[P * (P + 1) + (tt + P)];
       if (in_own || in_left) {
-        const double2 v = __ldg(&u2[n + tt]);
+        const double2 v = load_complex_ro<PAIR>(u, n + tt);
         sxr += cf * v.x;
         sxi += cf * v.y;
       }
@@ -108,7 +108,7 @@ __global__ void residual_noalloc_kernel(const __grid_constant__ NoallocArgs a, c
       if (in_own) cf += a.Kref[ay * (P + 1) + bb];
       if (in_below) cf += a.Kref[P * (P + 1) + (tt + P)];
       if (in_own || in_below) {
-        const double2 v = __ldg(&u2[n + (int64_t)tt * a.NXg]);
+        const double2 v = load_complex_ro<PAIR>(u, n + (int64_t)tt * a.NXg);
         syr += cf * v.x;
         syi += cf * v.y;
       }
@@ -120,7 +120,7 @@ __global__ void residual_noalloc_kernel(const __grid_constant__ NoallocArgs a, c
     const double cc = c[n];
     const double M = Wx * Wy / (cc * cc);
     const double H = (((J == 0 || J == a.NYg - 1) ? Wx : 0.0) + ((I == 0 || I == a.NXg - 1) ? Wy : 0.0)) / cc;
-    const double2 un = u2[n];
+    const double2 un = load_complex_ro<PAIR>(u, n);
     const double w = a.omega;
     const double Kur = Aur + w * H * un.y - w * w * M * un.x;
     const double Kui = Aui - w * H * un.x - w * w * M * un.y;
@@ -157,7 +157,8 @@ __global__ void residual_noalloc_kernel(const __grid_constant__ NoallocArgs a, c
 template <int P>
 void launch_na(const NoallocArgs& a, dim3 grd, const double* c, const double* b, const double* u, double* r,
                double* part, cudaStream_t st) {
-  residual_noalloc_kernel<P><<<grd, dim3(32, 8), 0, st>>>(a, c, b, u, r, part);
+  auto kern = is_pair_aligned(u) ? residual_noalloc_kernel<P, true> : residual_noalloc_kernel<P, false>;
+  kern<<<grd, dim3(32, 8), 0, st>>>(a, c, b, u, r, part);
 }
 
 }  // namespace

@@ -88,3 +88,39 @@ def test_residual_takes_arrays_at_any_double(hz, nx, ny, P, which):
     for a, c in zip(*out):
         assert np.any(a != 0.0) and np.array_equal(a, c)
     case.close()
+
+
+def test_older_step_calls_take_arrays_at_any_double(hz):
+    """The curved residual's u, the no-allocation residual and the lambda slot copies."""
+    import torch
+
+    wl = _wl(12, 8, 4, 4, 3)
+    case, pr = _pair(hz, wl)
+    m = pr.mesh
+    rng = np.random.default_rng(1)
+    b, u = (_dev(rng.standard_normal(2 * case.n)) for _ in range(2))
+    c = torch.from_numpy(np.ascontiguousarray(case.c.ravel())).cuda()
+    lam = _dev(_rand_lam(pr, 2))
+    slots = torch.tensor([[0, 1], [4, 2], [m.L, 0], [2, 3]], dtype=torch.int32, device="cuda")
+    out = []
+    for off in (False, True):
+        move = _off if off else (lambda t: t)
+        r, nrm = _zeros(2 * case.n, off), _zeros(2, False)
+        hz.hz_residual_noalloc(case.mesh, wl.omega, c, move(b), move(u), r, nrm)
+        buf, back = _zeros(2 * 4 * m.NE, off), _zeros(lam.numel(), off)
+        hz.hz_lambda_gather(case.pr, slots, 4, move(lam), buf)
+        hz.hz_lambda_scatter(case.pr, slots, 4, buf, back)
+        torch.cuda.synchronize()
+        out.append([t.cpu().numpy() for t in (r, nrm, buf, back)])
+    xy = hz.hz_mesh_node_coords(case.mesh)
+    xy[:, 0] += 0.02 * np.sin(np.pi * xy[:, 0]) * np.sin(np.pi * xy[:, 1])
+    hz.hz_problem_set(case.pr, hz.HZ_NODE_COORDS, xy)
+    for k, off in enumerate((False, True)):
+        move = _off if off else (lambda t: t)
+        r, nrm = _zeros(2 * case.n, off), _zeros(2, False)
+        hz.hz_residual(case.pr, move(b), move(u), r, nrm)
+        torch.cuda.synchronize()
+        out[k] += [r.cpu().numpy(), nrm.cpu().numpy()]
+    for p, q in zip(*out):
+        assert np.any(p != 0.0) and np.array_equal(p, q)
+    case.close()
