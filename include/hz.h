@@ -68,7 +68,7 @@ typedef enum {
   HZ_ERR_TIMEOUT = 6,     /* a wait ran out (server poll) */
   HZ_ERR_BUSY = 7,        /* admission refused: HBM budget or queue full */
   HZ_ERR_NOT_FOUND = 8,   /* unknown ticket */
-  HZ_ERR_INTERNAL = 9,
+  HZ_ERR_INTERNAL = 9,    /* a bug, or a sweep kernel whose blocks could not exchange their data */
   HZ_ERR_UNSUPPORTED = 10 /* a size or degree outside the compiled kernels */
 } hz_status;
 
@@ -292,7 +292,11 @@ HZ_API hz_status hz_prepare(hz_problem pr, int32_t nt, void* stream);
  * and lam_in, run wh_iters WaveHoltz iterations (wh_tol as in
  * hz_solve_opts), write lam_out (lambda vector) and, if u_sub is not NULL,
  * the subdomain solutions (L x nly x nlx complex, nly = sub_ny*P+1,
- * nlx = sub_nx*P+1, subdomain-major).  precision: hz_precision of the loop. */
+ * nlx = sub_nx*P+1, subdomain-major).  precision: hz_precision of the loop.
+ * The call does not wait for the device, so its status says nothing of the
+ * values: should a subdomain's thread blocks fail to exchange their data
+ * within about a second, its u_sub and the lam_out slots that it sends are
+ * NaN (solves: HZ_ERR_INTERNAL). */
 HZ_API hz_status hz_sweep(hz_problem pr, int32_t precision, int32_t nt, int32_t wh_iters, double wh_tol,
                    const double* lam_in, double* lam_out, const double* rhs, double* u_sub, void* stream);
 

@@ -95,7 +95,7 @@ struct SweepArgs {
   double* u_sub;        // [L][nly][nlx] complex or null
   int* wh_iter_max;
   unsigned long long* wh_iter_sum;  // sum over subdomains of WaveHoltz iterations
-  int* flags;           // bit 0: non-finite value seen
+  int* flags;           // bit 0: non-finite value seen; bit 1: the exchange inside a cluster timed out
   const double* u0;     // [L][nly][nlx] complex or null: WaveHoltz starts from it instead of zero
   // rank-local sweeps (hz_sweep_rect): with rect_w > 0 the launch covers the
   // rect_w x (count / rect_w) subdomains of the grid starting at subdomain

@@ -674,6 +674,13 @@ struct Ctx {
   int64_t n2;  // doubles in a lambda vector
 };
 
+// The sweep kernels' flag word.
+hz_status check_flags(int f) {
+  if (f & 2) return fail(HZ_ERR_INTERNAL, "the exchange inside a thread-block cluster of the subdomain sweep timed out");
+  if (f & 1) return fail(HZ_ERR_DIVERGED, "non-finite values in the subdomain solve (time step too large?)");
+  return HZ_OK;
+}
+
 // Reads nd doubles from device small-buffer offset 0 and the flag words.
 hz_status fetch(Ctx& c, int nd, double* host, int* flags_host) {
   Problem& pr = c.pr;
@@ -683,7 +690,7 @@ hz_status fetch(Ctx& c, int nd, double* host, int* flags_host) {
   HZ_CUDA(cudaStreamSynchronize(c.st));
   std::memcpy(host, pr.hsmall.ptr, (size_t)nd * sizeof(double));
   std::memcpy(flags_host, static_cast<char*>(pr.hsmall.ptr) + 4096 * sizeof(double), 16);
-  if (flags_host[0] & 1) return fail(HZ_ERR_DIVERGED, "non-finite values in the subdomain solve (time step too large?)");
+  HZ_TRY(check_flags(flags_host[0]));
   for (int k = 0; k < nd; ++k)
     if (!std::isfinite(host[k])) return fail(HZ_ERR_DIVERGED, "non-finite value in the outer iteration");
   return HZ_OK;
@@ -902,7 +909,7 @@ hz_status dd_solve(Ctx& c, const double* rhs, double* u) {
           const double* hslot = hh + (size_t)j * (CS + 4);
           int fl[4];
           std::memcpy(fl, hslot + CS, 16);
-          if (fl[0] & 1) return fail(HZ_ERR_DIVERGED, "non-finite values in the subdomain solve (time step too large?)");
+          HZ_TRY(check_flags(fl[0]));
           c.rep.gmres_iters++;
           for (int i = 0; i <= j; ++i)
             H[(size_t)i * m + j] = two_pass ? cplx(hslot[2 * i] + hslot[2 * (m + 2) + 2 * i],

@@ -410,6 +410,7 @@ struct TileArgs {
   int spw, gs;    // FUSE: subdomains per warp, lanes per subdomain
   int wm;         // main warps (not FUSE)
   int offB;       // first edge lane of chain B
+  int mute;       // clusters (tests): 1: the second slab's first row goes nowhere
   double wx[kMaxP], wy[kMaxP];  // lumped weight of node a (a = 0: shared by two elements)
 };
 
@@ -419,17 +420,19 @@ struct TileArgs {
 enum Role { kBoth = 0, kTiles = 1, kChains = 2 };
 
 struct TolShared {
-  unsigned long long mbar[2][4];  // clusters: arrivals by step parity
+  unsigned long long mbar[2][2][4];  // clusters: arrivals by step parity; the same, seen by nobody
   // tolerance mode: per-warp and per-CTA partial norms, the decision
   double red[32][2];
   double part[2];
   int stop;
+  int gave_up;  // clusters: a wait for a neighbouring slab's data ran out
 };
 
 // ---- exchange between the slabs of a cluster.  A cluster barrier per step
 // costs every warp a release fence and the wait for the slowest CTA; here only
 // the warps at a slab's ends wait, for the bytes that the neighbouring slab
-// stores straight into their buffers (st.async counts them on an mbarrier):
+// stores straight into their buffers (st.async counts them on an mbarrier,
+// where the sender has announced them):
 // 144 subdomains of 129 x 129 nodes, P = 4: 754 us with a cluster barrier per
 // step (arrival and wait apart), 652 us; 9 of 97 x 97, P = 3: 140, 103 us.
 // Barriers by step parity and by what arrives: a row of T (from the slab
@@ -442,17 +445,25 @@ __device__ __forceinline__ unsigned peer_addr(unsigned addr, int rank) {
   return r;
 }
 __device__ __forceinline__ void mbar_init(unsigned mb) { asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(mb) : "memory"); }
+// The sender announces its bytes on the neighbour's barrier, which is the
+// barrier's one arrival of the step.  (The receiver may not: once it stops
+// waiting it would arrive on a barrier whose phase has not ended.)  Relaxed:
+// the bytes order themselves, a release here costs 60%.
 __device__ __forceinline__ void mbar_expect(bool on, unsigned mb, unsigned bytes) {
   asm volatile(
-      "{ .reg .pred q; .reg .b64 t; setp.ne.u32 q, %0, 0; @q mbarrier.arrive.expect_tx.shared::cta.b64 t, [%1], %2; }" ::"r"(
+      "{ .reg .pred q; setp.ne.u32 q, %0, 0; @q mbarrier.arrive.expect_tx.relaxed.cluster.shared::cluster.b64 _, [%1], %2; }" ::"r"(
           (unsigned)on),
       "r"(mb), "r"(bytes)
       : "memory");
 }
-// Waits for the phase; false after about a second (the caller records it and
-// stops waiting: a slab that never answers must not hang the device).
+// Waits for the phase; false after about a second and kLateLooks more looks
+// (the clock also runs while the slabs are not scheduled).  The caller then
+// stops waiting and the sweep's results are void: a slab that never answers
+// must not hang the device.
+constexpr int kLateLooks = 64;
 __device__ __forceinline__ bool mbar_wait(unsigned mb, unsigned phase) {
   const long long t0 = clock64();
+  int late = 0;
   do {
     unsigned ok;
     asm volatile(
@@ -461,7 +472,8 @@ __device__ __forceinline__ bool mbar_wait(unsigned mb, unsigned phase) {
         : "r"(mb), "r"(phase)
         : "memory");
     if (ok) return true;
-  } while (clock64() - t0 < 2000000000LL);
+    if (clock64() - t0 > 2000000000LL) ++late;
+  } while (late < kLateLooks);
   return false;
 }
 
@@ -613,12 +625,17 @@ __device__ __forceinline__ void tile_body(const TileArgs& x, unsigned char* smem
   if constexpr (CLUS) {
     mb0 = smem_addr(ts->mbar);
     if (threadIdx.x == 0) {
-      for (int k = 0; k < 8; ++k) mbar_init(mb0 + 8 * k);
+      ts->gave_up = 0;
+      for (int k = 0; k < 16; ++k) mbar_init(mb0 + 8 * k);
       asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (!firstC) {
       mbP = peer_addr(mb0, rk - 1);
       smP = peer_addr(smem_addr(sm), rk - 1);
+      if (MAIN && x.mute && rk == 1) {  // tests: the second slab's first row goes nowhere
+        mbP = mb0 + 64;
+        smP = smem_addr(sm);
+      }
     }
     if (!lastC) {
       mbN = peer_addr(mb0, rk + 1);
@@ -643,7 +660,7 @@ __device__ __forceinline__ void tile_body(const TileArgs& x, unsigned char* smem
   const bool firsty = by == 0 && firstC;
   // slabs of a cluster: the slab before takes this one's first row, the next
   // one the T of its last band; the warps that hold these bands wait for the
-  // neighbours' in turn, their first thread announces the bytes
+  // neighbours' in turn, the thread of a band's first tile announces its bytes
   const bool sendPrev = live && by == 0 && !firstC, sendNext = live && by == nb - 1 && !lastC;
   const int w0 = (int)(threadIdx.x & ~31u);  // the warp's first thread: its bands are w0 / LX .. (w0 + 31) / LX
   const bool waitPrev = MAIN && CLUS && !firstC && w0 == 0;
@@ -825,16 +842,12 @@ __device__ __forceinline__ void tile_body(const TileArgs& x, unsigned char* smem
           if (inA && lastE && !lastC) RB::st_async1(smN + z * (y.tax + cur), eT, mbN + 8 * (4 * cur + kChainPrev));
         }
       }
-      if constexpr (CLUS) {  // what the neighbours will store in this step (predicated: no divergence here)
-        const unsigned mb = mb0 + 32 * cur;
-        if constexpr (MAIN) {
-          mbar_expect(waitPrev && lane == 0, mb + 8 * kTilePrev, sxe * RB::kBytes);
-          mbar_expect(waitNext && lane == 0, mb + 8 * kTileNext, sxe * RB::kBytes);
-        }
-        if constexpr (CHAIN) {
-          mbar_expect(chainPrev && lane == 0, mb + 8 * kChainPrev, sizeof(Real));
-          mbar_expect(chainNext && lane == 0, mb + 8 * kChainNext, sizeof(Real));
-        }
+      if constexpr (CLUS) {  // what this slab stores in this step (predicated: no divergence here)
+        const unsigned bytes = MAIN ? sxe * RB::kBytes : sizeof(Real);
+        mbar_expect(MAIN ? sendPrev && bx == 0 : inA && e == 0 && !firstC,
+                    mbP + 8 * (4 * cur + (MAIN ? kTileNext : kChainNext)), bytes);
+        mbar_expect(MAIN ? sendNext && bx == 0 : inA && lastE && !lastC,
+                    mbN + 8 * (4 * cur + (MAIN ? kTilePrev : kChainPrev)), bytes);
       }
       const V ct = bc<V>((Real)tb.x), st = bc<V>((Real)tb.y), kz = bc<V>((Real)tb.z), kw = bc<V>((Real)tb.w);
       // ---- the part of the stiffness that the tile's own nodes give:
@@ -1099,6 +1112,26 @@ __device__ __forceinline__ void tile_body(const TileArgs& x, unsigned char* smem
     }
   }
 
+  if constexpr (CLUS) {
+    if (!answered)
+      for (int k = 0; k < CL; ++k) *cluster.map_shared_rank(&ts->gave_up, k) = 1;
+    cluster.sync();  // the neighbours' last pushes have landed, and word of waits that ran out
+    if (ts->gave_up) {
+      // No result rather than a wrong one: NaN in the subdomain's solution
+      // and in what it sends.  A push that nobody waited for may still be
+      // under way: a microsecond's work, given a hundred before this CTA ends.
+      const Real nan = Real(__int_as_float(0x7fffffff));
+#pragma unroll
+      for (int r = 0; r < P; ++r)
+#pragma unroll
+        for (int c = 0; c < P; ++c) v[r][c].a = v[r][c].b = bc<V>(nan);
+#pragma unroll
+      for (int q = 0; q <= P; ++q) ev[q].a = ev[q].b = nan;
+      for (const long long t0 = clock64(); clock64() - t0 < 200000;) {
+      }
+      if (threadIdx.x == 0) atomicOr(a.flags, 2);
+    }
+  }
   // ---- outputs
   bool bad = false;
   auto out = [&](int i, int j, Real re, Real im) {
@@ -1118,7 +1151,7 @@ __device__ __forceinline__ void tile_body(const TileArgs& x, unsigned char* smem
   for (int q = 0; q <= P; ++q)
     if (q < P ? inE : corner)
       out(inA ? nlx - 1 : eB * P + q, inA ? row0 + e * P + q : nly - 1, ev[q].a, ev[q].b);
-  if (bad || (CLUS && !answered)) atomicOr(a.flags, 1);  // a silent neighbour is reported as a failed solve
+  if (bad) atomicOr(a.flags, 1);
   if (t == 0 && have && firstC && a.wh_iter_max) {
     atomicMax(a.wh_iter_max, m_done);
     atomicAdd(a.wh_iter_sum, (unsigned long long)m_done);
@@ -1127,8 +1160,7 @@ __device__ __forceinline__ void tile_body(const TileArgs& x, unsigned char* smem
   // their last reads lie behind the barrier below), so that every thread
   // takes entries of the transmission update.  W, E: local rows; S, N: columns
   if (FUSE) __syncwarp();
-  else if (CLUS) cluster.sync();  // the neighbours' last pushes have landed
-  else block_bar();
+  else if (!CLUS) block_bar();  // (clusters: the barrier above)
   const int rowsC = nb * RH + (lastC ? 1 : 0);  // node rows of this slab
   const int nrow = nb * RH + 1;
   Real* uW = sm + y.tw;       // [rows][2]

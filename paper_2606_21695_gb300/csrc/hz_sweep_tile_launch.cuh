@@ -2,6 +2,8 @@
 // precision: the tile grid, the slabs and the launch shape by subdomain size.
 #pragma once
 
+#include <cstdlib>
+
 #include "hz_sweep_tile.cuh"
 
 namespace hz {
@@ -27,6 +29,8 @@ hz_status launch_tile_iso(const SweepArgs& a0, int count, cudaStream_t st, int* 
     x.wx[k] = a0.hx2 * wk;
     x.wy[k] = a0.hy2 * wk;
   }
+  const char* mute = std::getenv("HZ_TILE_MUTE");  // 1: data that never comes (tests)
+  x.mute = mute ? std::atoi(mute) : 0;
   const bool tol = a0.wh_tol > 0.0;
   const int lanes = x.LX * x.nbt, need = lanes > sxe + sye ? lanes : sxe + sye;
   if (need <= 32) {  // the whole subdomain in (part of) one warp

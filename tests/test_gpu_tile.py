@@ -121,3 +121,36 @@ def test_curved_tile_sweep_matches_oracle(hz, monkeypatch, nx, ny, sx, sy, P):
         _, ref_u, _ = pr.sweep(lam, None, nt, 30, wh_tol=1e-3, want_u=True)
         assert _rel(u, ref_u) < 1e-2
         case.close()
+
+
+@pytest.mark.parametrize("nx,ny,sx,sy,P,shape,precision", [
+    (24, 22, 12, 22, 3, 1, "fp32"),   # two slabs: the two that wait for each other
+    (64, 32, 32, 32, 3, 2, "fp32"),
+    (64, 32, 32, 32, 4, 1, "fp32"),   # more than two: slabs that saw nothing amiss themselves
+    (64, 32, 32, 32, 3, 1, "fp64"),
+])
+def test_cluster_exchange_that_runs_out_gives_nan_and_an_error(hz, monkeypatch, nx, ny, sx, sy, P, shape, precision):
+    """One slab of every subdomain withholds a row that its neighbour waits for, so that the wait runs out (after
+    about a second): the sweep ends with NaN in every subdomain's solution and in all that it sends, a solve with
+    HZ_ERR_INTERNAL; without that, the same problem is swept and solved as ever."""
+    _force(monkeypatch, shape)
+    case, pr = _pair(hz, _wl(nx, ny, sx, sy, P))
+    prec = hz.HZ_FP32_REFINE if precision == "fp32" else hz.HZ_FP64
+    nt, lam = hz.hz_problem_nt(case.pr), _rand_lam(pr, 9)
+    opts = hz.hz_default_opts(precision=prec, tol=1e-6)
+    ref_l, ref_u = _run_sweep(hz, case, pr, prec, nt, 2, lam, False)
+    for wh_tol in (0.0, 1e-3):
+        with monkeypatch.context() as mp:
+            mp.setenv("HZ_TILE_MUTE", "1")
+            got_l, got_u = _run_sweep(hz, case, pr, prec, nt, 2, lam, False, wh_tol=wh_tol)
+            assert np.all(np.isnan(got_u))
+            assert np.all(np.isnan(got_l[lam != 0]))  # every interface slot
+            if wh_tol == 0.0:
+                with pytest.raises(hz.HzError) as e:
+                    hz.hz_solve(case.pr, opts, n=case.n)
+                assert e.value.status == hz.HZ_ERR_INTERNAL
+    got_l, got_u = _run_sweep(hz, case, pr, prec, nt, 2, lam, False)
+    assert np.array_equal(got_u, ref_u) and np.array_equal(got_l, ref_l)
+    st, _, rep = hz.hz_solve(case.pr, opts, n=case.n)
+    assert st == hz.HZ_OK and rep["rel_residual"] <= 1e-6
+    case.close()
