@@ -250,11 +250,14 @@ __global__ void __launch_bounds__(ONE ? 32 : 256) sweep_mapped_tile_kernel(const
 #pragma unroll
           for (int c = 0; c < M; ++c) A[q][c] = fmaf(x.D[k * M + c], f1[k], A[q][c]);
       }
-      // x neighbours, then the row sums to the y neighbours
+      // x neighbours (by rows of elements: the ends multiply what they get by
+      // zero, which may not be another subdomain's infinity or NaN), then the
+      // row sums to the y neighbours
+      const int width = ONE ? x.LX : 32;
 #pragma unroll
       for (int b = 0; b < M; ++b) {
-        const float fr = __shfl_down_sync(0xffffffffu, A[b][0], 1);
-        const float fl = __shfl_up_sync(0xffffffffu, A[b][P], 1);
+        const float fr = __shfl_down_sync(0xffffffffu, A[b][0], 1, width);
+        const float fl = __shfl_up_sync(0xffffffffu, A[b][P], 1, width);
         A[b][0] = fmaf(ml, fl, A[b][0]);
         A[b][P] = fmaf(mr, fr, A[b][P]);
       }

@@ -480,7 +480,7 @@ __device__ __forceinline__ bool mbar_wait(unsigned mb, unsigned phase) {
 // Block barrier met by warps at different places of the program (the roles).
 __device__ __forceinline__ void block_bar() { asm volatile("bar.sync 0;" ::: "memory"); }
 
-template <typename Real, int P, int H, int ROLE, bool SRC, bool ISO, bool CLUS>
+template <typename Real, int P, int H, int ROLE, bool SHARED, bool SRC, bool ISO, bool CLUS>
 __device__ __forceinline__ void tile_body(const TileArgs& x, unsigned char* smem_raw, TolShared* ts) {
   constexpr bool FUSE = ROLE == kBoth, MAIN = ROLE != kChains, CHAIN = ROLE != kTiles;
   using V = typename VecT<Real, H>::V;
@@ -812,6 +812,9 @@ __device__ __forceinline__ void tile_body(const TileArgs& x, unsigned char* smem
         for (int r = 0; r < P; ++r) {
           xe[r] = shfl_down1(s[r][0].a);
           xt[r] = shfl_up1(Tx[r]);
+          // The first column multiplies what it gets by zero; in a warp of
+          // several subdomains that may be another one's infinity or NaN.
+          if (SHARED && firstx) xt[r] = bc<V>(Real(0));
         }
 #pragma unroll
         for (int h = 0; h < H; ++h) {
@@ -1232,15 +1235,18 @@ __device__ __forceinline__ void tile_body(const TileArgs& x, unsigned char* smem
   }
 }
 
-template <typename Real, int P, int H, bool FUSE, bool SRC, bool ISO, bool CLUS, int MAXT>
+// LANES: lanes of a one-warp subdomain are 1 the whole warp, 2 a part of it;
+// 0: more than one warp.  (1 and 2 apart: selecting zeros costs the benchmark's
+// one-warp subdomains 2.7%, those that share a warp 0.5%.)
+template <typename Real, int P, int H, int LANES, bool SRC, bool ISO, bool CLUS, int MAXT>
 __global__ void __launch_bounds__(MAXT) sweep_tile_kernel(const __grid_constant__ TileArgs x) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  if constexpr (FUSE) {
-    tile_body<Real, P, H, kBoth, SRC, ISO, CLUS>(x, smem_raw, nullptr);
+  if constexpr (LANES > 0) {
+    tile_body<Real, P, H, kBoth, LANES == 2, SRC, ISO, CLUS>(x, smem_raw, nullptr);
   } else {
     __shared__ TolShared ts;
-    if ((int)(threadIdx.x >> 5) < x.wm) tile_body<Real, P, H, kTiles, SRC, ISO, CLUS>(x, smem_raw, &ts);
-    else tile_body<Real, P, H, kChains, SRC, ISO, CLUS>(x, smem_raw, &ts);
+    if ((int)(threadIdx.x >> 5) < x.wm) tile_body<Real, P, H, kTiles, false, SRC, ISO, CLUS>(x, smem_raw, &ts);
+    else tile_body<Real, P, H, kChains, false, SRC, ISO, CLUS>(x, smem_raw, &ts);
   }
 }
 

@@ -40,7 +40,8 @@ hz_status launch_tile_iso(const SweepArgs& a0, int count, cudaStream_t st, int* 
     x.offB = sye;
     const Lay y = make_lay<P, Real>(H, x.LX, x.nb, x.gs, SRC, tol);
     const size_t smem = (size_t)x.spw * y.total * sizeof(Real);
-    auto kern = sweep_tile_kernel<Real, P, H, true, SRC, ISO, false, 32>;
+    auto kern = x.spw > 1 ? sweep_tile_kernel<Real, P, H, 2, SRC, ISO, false, 32>
+                          : sweep_tile_kernel<Real, P, H, 1, SRC, ISO, false, 32>;
     if (smem > 48 * 1024) HZ_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem));
     kern<<<(count + x.spw - 1) / x.spw, 32, smem, st>>>(x);
     note_launch();
@@ -60,8 +61,8 @@ hz_status launch_tile_iso(const SweepArgs& a0, int count, cudaStream_t st, int* 
     const Lay y = make_lay<P, Real>(H, x.LX, x.nb, threads, SRC, tol);
     const size_t smem = (size_t)y.total * sizeof(Real);
     if (smem > kMaxSmem) continue;
-    auto kern = CL > 1 ? sweep_tile_kernel<Real, P, H, false, SRC, ISO, true, MAXT>
-                       : sweep_tile_kernel<Real, P, H, false, SRC, ISO, false, MAXT>;
+    auto kern = CL > 1 ? sweep_tile_kernel<Real, P, H, 0, SRC, ISO, true, MAXT>
+                       : sweep_tile_kernel<Real, P, H, 0, SRC, ISO, false, MAXT>;
     if (smem > 48 * 1024) HZ_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem));
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)(count * CL));

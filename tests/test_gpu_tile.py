@@ -154,3 +154,41 @@ def test_cluster_exchange_that_runs_out_gives_nan_and_an_error(hz, monkeypatch, 
     st, _, rep = hz.hz_solve(case.pr, opts, n=case.n)
     assert st == hz.HZ_OK and rep["rel_residual"] <= 1e-6
     case.close()
+
+
+@pytest.mark.parametrize("curved", [False, True])
+@pytest.mark.parametrize("nx,ny,sx,sy,P,shape", [
+    (3, 3, 1, 1, 2, 1),     # 16 subdomains per warp (curved: 32)
+    (12, 4, 4, 4, 3, 1),    # 2 per warp, all lanes in use
+    (12, 4, 4, 4, 3, 2),    # 4 per warp
+    (9, 9, 3, 3, 4, 1),     # idle lanes between the subdomains
+    (16, 16, 8, 8, 3, 2),   # one subdomain per warp
+])
+def test_non_finite_subdomain_leaves_the_others_alone(hz, monkeypatch, nx, ny, sx, sy, P, shape, curved):
+    """What one subdomain receives (NaN, infinity, a value beyond FP32) shows in its own solution and in what it
+    sends, and nowhere else: every other subdomain's result is that of the clean sweep, bit for bit, also where the
+    subdomains share a warp."""
+    _force(monkeypatch, shape)
+    case, pr = _pair(hz, _wl(nx, ny, sx, sy, P))
+    if curved:
+        xy = hz.hz_mesh_node_coords(case.mesh)
+        xy[:, 0] += 0.02 * np.sin(np.pi * xy[:, 0]) * np.sin(np.pi * xy[:, 1])
+        hz.hz_problem_set(case.pr, hz.HZ_NODE_COORDS, xy)
+    nt, lam, L = hz.hz_problem_nt(case.pr), _rand_lam(pr, 10), pr.mesh.L
+    ref_l, ref_u = _run_sweep(hz, case, pr, hz.HZ_FP32_REFINE, nt, 2, lam, False)
+    for l in range(L):
+        for value in (np.nan, np.inf, 1e300):
+            bad = lam.copy()
+            e = next(e for e in range(4) if pr.nbr[l, e] >= 0)
+            bad[l, e, 1] = value
+            got_l, got_u = _run_sweep(hz, case, pr, hz.HZ_FP32_REFINE, nt, 2, bad, False)
+            others = [k for k in range(L) if k != l]
+            assert not np.all(np.isfinite(got_u[l]))
+            assert np.array_equal(got_u[others], ref_u[others]), (l, value)
+            sent = np.zeros(lam.shape[:2], bool)  # slots that subdomain l writes
+            sent[l] = pr.nbr[l] < 0
+            for q in range(4):
+                if pr.nbr[l, q] >= 0:
+                    sent[pr.nbr[l, q], q ^ 1] = True
+            assert np.array_equal(got_l[~sent], ref_l[~sent]), (l, value)
+    case.close()
