@@ -654,8 +654,15 @@ __device__ __forceinline__ void tile_body(const TileArgs& x, unsigned char* smem
   const Real cpi = Real(a.cpi), spi = Real(a.spi), scale = Real(a.two_over_nt);
   const V vsig = bc<V>(sigma);
   const double rys = (a.hx2 / a.hy2) * (a.hx2 / a.hy2);  // (4 / hy^2) / (4 / hx^2)
+  // FP32: rys in two terms, in every y term of a row, or its rounding is left
+  // over where the row should annihilate constants, at every time step with
+  // the same sign (P = 4, N_t = 464, rys 0.99 half units off: error 1.9e-6
+  // with one term in the partial sum T, 5.6e-7 with two everywhere)
+  constexpr bool kLow = sizeof(Real) == 4;
   const V ry = bc<V>((Real)rys), ryl = bc<V>((Real)(rys - (double)(Real)rys));
   const Real rye = lo(ry), ryle = lo(ryl);
+  auto scale_y = [&](V v) { return kLow ? vfma(ry, v, vmul(ryl, v)) : vmul(ry, v); };
+  auto scale_ye = [&](Real v) { return kLow ? rye * v + ryle * v : rye * v; };
   const bool firstx = bx == 0, lastx = live && bx == sxe - 1;
   const bool firsty = by == 0 && firstC;
   // slabs of a cluster: the slab before takes this one's first row, the next
@@ -705,7 +712,7 @@ __device__ __forceinline__ void tile_body(const TileArgs& x, unsigned char* smem
   // the subdomain's first column and row: twice the own part, nothing received
   const Real mx = firstx ? Real(2) : Real(1), rx = firstx ? Real(0) : Real(1);
   const V my = half_of<H, V>(firsty ? Real(2) : Real(1), Real(1));
-  const V rry = half_of<H, V>(firsty ? Real(0) : (Real)rys, (Real)rys);
+  const V rry = half_of<H, V>(firsty ? Real(0) : rye, rye), rryl = half_of<H, V>(firsty ? Real(0) : ryle, ryle);
 
   Pair<V> s[P][P], v[P][P];         // p, p-dot; the filter sums
   Pair<Real> es[P + 1], ev[P + 1];  // the chain's
@@ -885,7 +892,7 @@ __device__ __forceinline__ void tile_body(const TileArgs& x, unsigned char* smem
           }
           if (!ISO) {  // (hx/hy)^2, its FP32 rounding made up by a second term
 #pragma unroll
-            for (int c = 0; c < P; ++c) Y[c] = vfma(ry, Y[c], vmul(ryl, Y[c]));
+            for (int c = 0; c < P; ++c) Y[c] = scale_y(Y[c]);
           }
           A[r][0] = vfma(K.diag(), s[r][0].a, Y[0]);
           if (P > 1) A[r][0] = vfma(bc<V>(mx), X[0], A[r][0]);
@@ -942,8 +949,10 @@ __device__ __forceinline__ void tile_body(const TileArgs& x, unsigned char* smem
 #pragma unroll
         for (int c = 0; c < P; ++c) {
           ye[c] = half_of<H, V>(H == 2 ? hi(s[0][c].a) : ey[c], ey[c]);
-          if (!ISO) ye[c] = vfma(ry, ye[c], vmul(ryl, ye[c]));
-          A[0][c] = vfma(rry, half_of<H, V>(ty[c], lo(Ty[c])), A[0][c]);
+          if (!ISO) ye[c] = scale_y(ye[c]);
+          const V T = half_of<H, V>(ty[c], lo(Ty[c]));
+          if (!ISO && kLow) A[0][c] = vfma(rryl, T, A[0][c]);
+          A[0][c] = vfma(rry, T, A[0][c]);
         }
         const V mkP = vmul(bc<V>(mx), K.own(P)), myP = vmul(my, K.own(P));
 #pragma unroll
@@ -982,14 +991,14 @@ __device__ __forceinline__ void tile_body(const TileArgs& x, unsigned char* smem
           }
           const Real C = Ke.diag() * es[q].a + Real(2) * cr[q];
           // the y sum is the chain's own on chain A, the one across it on chain B
-          const Real Ac = ISO ? S + C : inA ? C + (rye * S + ryle * S) : S + (rye * C + ryle * C);
+          const Real Ac = ISO ? S + C : inA ? C + scale_ye(S) : S + scale_ye(C);
           es[q].b = eal[q] * es[q].b + ebet[q] * Ac + ebr[q] * ec + ebi[q] * esn;
           accumulate(ev[q], (Real)tb.z, (Real)tb.w, es[q]);
         }
         // the corner (zero coefficients elsewhere)
         const Real d = Ke.diag() * es[P].a;
         const Real Y = d + Real(2) * eT;
-        const Real Ac = (d + Real(2) * ca) + (ISO ? Y : rye * Y + ryle * Y);
+        const Real Ac = (d + Real(2) * ca) + (ISO ? Y : scale_ye(Y));
         es[P].b = eal[P] * es[P].b + ebet[P] * Ac + ebr[P] * ec + ebi[P] * esn;
         accumulate(ev[P], (Real)tb.z, (Real)tb.w, es[P]);
       }

@@ -192,3 +192,24 @@ def test_non_finite_subdomain_leaves_the_others_alone(hz, monkeypatch, nx, ny, s
                     sent[pr.nbr[l, q], q ^ 1] = True
             assert np.array_equal(got_l[~sent], ref_l[~sent]), (l, value)
     case.close()
+
+
+def test_element_ratio_rounding_does_not_build_up(hz, monkeypatch):
+    """Non-square elements: (hx / hy)^2 times an assembled row that annihilates constants has to annihilate them too.
+    A ratio rounded to FP32 in some of the row's terms leaves an error that every time step adds with the same sign
+    (relative to the wave's own term it grows with N_t^2), where the rounding of the state grows with its square
+    root.  So at a low frequency (N_t of several hundred) a badly rounded ratio, (56/79)^2, may not be worse than an
+    exactly representable one, (3/4)^2, by more than the scatter of the state's rounding (a factor of 3)."""
+    err = {}
+    for name, ratio in (("exact", 3 / 4), ("rounded", 56 / 79)):  # hx / hy
+        for shape, P in ((1, 3), (2, 3), (1, 4)):
+            _force(monkeypatch, shape)
+            case, pr = _pair(hz, _wl(32, 16, 16, 16, P, omega=4.0, kind="const", box=(0.0, 1.0, 0.0, 0.5 / ratio)))
+            nt = hz.hz_problem_nt(case.pr)
+            lam = _rand_lam(pr, 13)
+            _, u = _run_sweep(hz, case, pr, hz.HZ_FP32_REFINE, nt, 8, lam, False)
+            _, ref, _ = pr.sweep(lam, None, nt, 8, want_u=True)
+            err[name, shape, P] = _rel(u, ref)
+            case.close()
+    for shape, P in ((1, 3), (2, 3), (1, 4)):
+        assert err["rounded", shape, P] < 3 * err["exact", shape, P], (err, nt)
