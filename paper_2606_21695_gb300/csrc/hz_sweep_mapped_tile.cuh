@@ -326,7 +326,9 @@ __global__ void __launch_bounds__(ONE ? 32 : 256) sweep_mapped_tile_kernel(const
       NormAcc acc;
       float big = 0.f;
 #pragma unroll
-      for (int k = 0; k < N2; ++k) big = fmaxf(big, fmaxf(fabsf(v[k / M][k % M].x), fabsf(v[k / M][k % M].y)));
+      for (int k = 0; k < N2; ++k)
+        big = fmaxf(fmaxf(big, fmaxf(fabsf(v[k / M][k % M].x), fabsf(v[k / M][k % M].y))),
+                    fmaxf(fabsf(st[(2 * k) * nthr + t]), fabsf(st[(2 * k + 1) * nthr + t])));
       acc.start(big);
 #pragma unroll
       for (int b = 0; b < M; ++b)
@@ -335,8 +337,7 @@ __global__ void __launch_bounds__(ONE ? 32 : 256) sweep_mapped_tile_kernel(const
           const int k = b * M + c;
           const float orr = st[(2 * k) * nthr + t], oi = st[(2 * k + 1) * nthr + t];
           if (live && (c < P || lastx) && (b < P || lasty)) {
-            acc.add(v[b][c].x, orr);
-            acc.add(v[b][c].y, oi);
+            acc.add(v[b][c], make_float2(orr, oi));
           }
           if (done) v[b][c] = make_float2(orr, oi);
         }

@@ -38,9 +38,9 @@
 // scheduler at 1024 one-warp subdomains).  Measured, 20 WaveHoltz iterations:
 // 1024 subdomains of 25 x 25 nodes, P = 3, N_t = 55: 1073 us with the one-warp
 // column kernel (hz_sweep_warp.cuh: 4 shuffles and 30 instructions per node row
-// and step), 565 us here; 16 of 17 x 17, P = 2, N_t = 79: 610, 168 us; 1024 of
+// and step), 570 us here; 16 of 17 x 17, P = 2, N_t = 79: 610, 157 us; 1024 of
 // 129 x 129, P = 4, N_t = 48: 59.8 ms with the cluster of warp bands, 108.6 ms
-// with the cluster kernel, 22.4 ms here.  A launch with clusters is a separate
+// with the cluster kernel, 20.7 ms here.  A launch with clusters is a separate
 // instantiation: its few branches per step alone cost the others 20 to 40%.
 //
 // Taken by size (tile_shape, tile_default in hz_sweep_tile_dispatch.cu):
@@ -253,6 +253,33 @@ struct Coef {
 // element's nodes move in one or two shared-memory instructions.
 template <int P, typename Real>
 struct RowBuf;
+// Shared-memory stores under a condition that never become branches: kernels of
+// several warps (the compiler's own choice costs 64 subdomains of 97 x 97 nodes,
+// P = 3, 218 us against 202; one-warp kernels schedule better with it).
+__device__ __forceinline__ unsigned smem_addr(const void* q) { return (unsigned)__cvta_generic_to_shared(q); }
+__device__ __forceinline__ void st_if(bool on, unsigned addr, float a) {
+  asm volatile("{ .reg .pred q; setp.ne.u32 q, %0, 0; @q st.shared.f32 [%1], %2; }" ::"r"((unsigned)on), "r"(addr), "f"(a)
+               : "memory");
+}
+__device__ __forceinline__ void st_if(bool on, unsigned addr, float a, float b) {
+  asm volatile("{ .reg .pred q; setp.ne.u32 q, %0, 0; @q st.shared.v2.f32 [%1], {%2, %3}; }" ::"r"((unsigned)on),
+               "r"(addr), "f"(a), "f"(b)
+               : "memory");
+}
+__device__ __forceinline__ void st_if(bool on, unsigned addr, float a, float b, float c, float d) {
+  asm volatile("{ .reg .pred q; setp.ne.u32 q, %0, 0; @q st.shared.v4.f32 [%1], {%2, %3, %4, %5}; }" ::"r"((unsigned)on),
+               "r"(addr), "f"(a), "f"(b), "f"(c), "f"(d)
+               : "memory");
+}
+__device__ __forceinline__ void st_if(bool on, unsigned addr, double a) {
+  asm volatile("{ .reg .pred q; setp.ne.u32 q, %0, 0; @q st.shared.f64 [%1], %2; }" ::"r"((unsigned)on), "r"(addr), "d"(a)
+               : "memory");
+}
+__device__ __forceinline__ void st_if(bool on, unsigned addr, double a, double b) {
+  asm volatile("{ .reg .pred q; setp.ne.u32 q, %0, 0; @q st.shared.v2.f64 [%1], {%2, %3}; }" ::"r"((unsigned)on),
+               "r"(addr), "d"(a), "d"(b)
+               : "memory");
+}
 template <int P>
 struct RowBuf<P, float> {
   static constexpr int kQ = P / 4 + (P % 4 == 3 ? 1 : 0);  // quads
@@ -266,6 +293,19 @@ struct RowBuf<P, float> {
           make_float4(at(v, 4 * f), at(v, 4 * f + 1), at(v, 4 * f + 2), at(v, 4 * f + 3));
     if (kP2) reinterpret_cast<float2*>(buf + 4 * kQ * n)[idx] = make_float2(at(v, 4 * kQ), at(v, 4 * kQ + 1));
     if (kP1) buf[4 * kQ * n + idx] = at(v, 4 * kQ);
+  }
+  template <bool PRED>
+  static __device__ __forceinline__ void st(bool on, float* buf, int n, int idx, const float (&v)[P]) {
+    if constexpr (!PRED) {
+      if (on) st(buf, n, idx, v);
+      return;
+    }
+    const unsigned b = smem_addr(buf);
+#pragma unroll
+    for (int f = 0; f < kQ; ++f)
+      st_if(on, b + 16 * (f * n + idx), at(v, 4 * f), at(v, 4 * f + 1), at(v, 4 * f + 2), at(v, 4 * f + 3));
+    if (kP2) st_if(on, b + 16 * kQ * n + 8 * idx, at(v, 4 * kQ), at(v, 4 * kQ + 1));
+    if (kP1) st_if(on, b + 16 * kQ * n + 4 * idx, at(v, 4 * kQ));
   }
   static __device__ __forceinline__ void ld(const float* buf, int n, int idx, float (&v)[P]) {
 #pragma unroll
@@ -313,6 +353,17 @@ struct RowBuf<P, double> {
 #pragma unroll
     for (int f = 0; f < kD; ++f) reinterpret_cast<double2*>(buf)[f * n + idx] = make_double2(v[2 * f], v[2 * f + 1]);
     if (P % 2) buf[2 * kD * n + idx] = v[P - 1];
+  }
+  template <bool PRED>
+  static __device__ __forceinline__ void st(bool on, double* buf, int n, int idx, const double (&v)[P]) {
+    if constexpr (!PRED) {
+      if (on) st(buf, n, idx, v);
+      return;
+    }
+    const unsigned b = smem_addr(buf);
+#pragma unroll
+    for (int f = 0; f < kD; ++f) st_if(on, b + 16 * (f * n + idx), v[2 * f], v[2 * f + 1]);
+    if (P % 2) st_if(on, b + 16 * kD * n + 8 * idx, v[P - 1]);
   }
   static __device__ __forceinline__ void ld(const double* buf, int n, int idx, double (&v)[P]) {
 #pragma unroll
@@ -438,7 +489,6 @@ struct TolShared {
 // Barriers by step parity and by what arrives: a row of T (from the slab
 // before), a row of p (from the one after), chain A's T and p.
 enum { kTilePrev = 0, kTileNext = 1, kChainPrev = 2, kChainNext = 3 };
-__device__ __forceinline__ unsigned smem_addr(const void* q) { return (unsigned)__cvta_generic_to_shared(q); }
 __device__ __forceinline__ unsigned peer_addr(unsigned addr, int rank) {
   unsigned r;
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
@@ -480,7 +530,7 @@ __device__ __forceinline__ bool mbar_wait(unsigned mb, unsigned phase) {
 // Block barrier met by warps at different places of the program (the roles).
 __device__ __forceinline__ void block_bar() { asm volatile("bar.sync 0;" ::: "memory"); }
 
-template <typename Real, int P, int H, int ROLE, bool SHARED, bool SRC, bool ISO, bool CLUS>
+template <typename Real, int P, int H, int ROLE, bool SHARED, bool SRC, bool ISO, bool CLUS, bool TOL>
 __device__ __forceinline__ void tile_body(const TileArgs& x, unsigned char* smem_raw, TolShared* ts) {
   constexpr bool FUSE = ROLE == kBoth, MAIN = ROLE != kChains, CHAIN = ROLE != kTiles;
   using V = typename VecT<Real, H>::V;
@@ -516,7 +566,8 @@ __device__ __forceinline__ void tile_body(const TileArgs& x, unsigned char* smem
   const bool corner = inA && lastC && e == nA - 1;
 
   using RB = RowBuf<P, Real>;
-  const Lay y = make_lay<P, Real>(H, LX, x.nb, nthr, SRC, a.wh_tol > 0.0);
+  const bool tol = TOL && a.wh_tol > 0.0;
+  const Lay y = make_lay<P, Real>(H, LX, x.nb, nthr, SRC, tol);
   const int ncol = x.nb * H + 1;  // elements of a column buffer
   Real* sm = reinterpret_cast<Real*>(smem_raw) + (FUSE ? grp * y.total : 0);
   const int64_t nn = (int64_t)nlx * nly;
@@ -676,7 +727,6 @@ __device__ __forceinline__ void tile_body(const TileArgs& x, unsigned char* smem
   const bool chainNext = CHAIN && CLUS && !lastC && (int)(threadIdx.x >> 5) == x.wm;
   bool answered = true;
   unsigned phase = 0;  // of the barriers of the current parity
-  const bool tol = a.wh_tol > 0.0;
   // the tile's nodes on the west column and the south row: alpha - 1 and
   // beta b in registers (zero on the other tiles: no branch in the time loop)
   V wal[P], wbr[P], wbi[P];
@@ -723,11 +773,15 @@ __device__ __forceinline__ void tile_body(const TileArgs& x, unsigned char* smem
 #pragma unroll
   for (int q = 0; q <= P; ++q) ev[q].a = ev[q].b = Real(0);
 
-  // Two steps per turn of the time loop, so that each parity's buffers are fixed
-  // offsets: 1024 subdomains of 25 x 25 nodes, P = 3: 602 us with one, 565 us.
-  // Not where it takes more registers than there are (P = 3 with a source: 52
-  // bytes spilled, P = 5: 96 to 256).
-  constexpr bool kTwo = FUSE && P <= 3 && !SRC;
+  // Several steps per turn of a one-warp kernel's time loop, an even number, so
+  // that each parity's buffers are fixed offsets.  1024 subdomains of 25 x 25
+  // nodes, P = 3, by 1 / 2 / 4 / 6 / 8 steps: 650 / 635 / 588 / 573 / 695 us; with
+  // a source by 1 / 2 / 4 / 6: 736 / 743 / 705 / 745; twice as many, not square, by
+  // 1 / 2 / 4 / 6: 452 / 413 / 382 / 461; the tolerance mode has its best at 2.
+  // P = 4 and 5 spill (96 to 256 bytes at P = 5).
+  constexpr bool kPairs = P == 3 && H == 2;
+  constexpr int kTurn = !FUSE || P > 3 ? 1 : !kPairs ? (SRC ? 1 : 2) : TOL ? 2 : ISO && !SRC ? 6 : 4;
+  constexpr bool kTwo = kTurn > 1;  // parity known at compile time
   int cur = 0, m_done = 0;
   bool done = false;  // tolerance met (FUSE: this lane group; else the whole subdomain)
   for (int m = 0; m < a.m_wh; ++m) {
@@ -771,7 +825,7 @@ __device__ __forceinline__ void tile_body(const TileArgs& x, unsigned char* smem
     }
     Tab tb = tab[1];
     if (kTwo) __syncwarp();  // the first step may write the buffers that the last iteration's last step read
-#pragma unroll (kTwo ? 2 : 1)
+#pragma unroll kTurn
     for (int nu = 1; nu < a.Nt; ++nu) {
       if (kTwo) cur = nu & 1;
       const Tab tn = tab[nu + 1];  // prefetch (the table has N_t + 1 entries)
@@ -799,10 +853,8 @@ __device__ __forceinline__ void tile_body(const TileArgs& x, unsigned char* smem
           p0[c] = lo(s[0][c].a);
           th[c] = hi(Ty[c]);
         }
-        if (live) {
-          RB::st(PY + by * y.row, LX, bx, p0);
-          RB::st(TY + (by + 1) * y.row, LX, bx, th);
-        }
+        RB::template st<!FUSE>(live, PY + byc * y.row, LX, bx, p0);
+        RB::template st<!FUSE>(live, TY + (byc + 1) * y.row, LX, bx, th);
         if constexpr (CLUS) {
           const unsigned z = sizeof(Real);
           if (sendPrev) RB::st_async(smP + z * (y.py + cur * pr_ + x.nb * y.row), LX, bx, p0, mbP + 8 * (4 * cur + kTileNext));
@@ -828,7 +880,7 @@ __device__ __forceinline__ void tile_body(const TileArgs& x, unsigned char* smem
           Real tv[P];
 #pragma unroll
           for (int r = 0; r < P; ++r) tv[r] = get<H>(Tx[r], h);
-          if (lastx) RB::st(TA, ncol, byc * H + h, tv);
+          RB::template st<!FUSE>(lastx, TA, ncol, byc * H + h, tv);
         }
       }
       if constexpr (CHAIN) {
@@ -842,9 +894,14 @@ __device__ __forceinline__ void tile_body(const TileArgs& x, unsigned char* smem
         Real tv[P];
 #pragma unroll
         for (int q = 0; q < P; ++q) tv[q] = es[q].a;
-        if (inE) RB::st(inB ? PY + nb * y.row : CP, en, ei, tv);
-        if (corner) *RB::first(CP, nA) = es[P].a;
-        if (inB && lastE) *RB::first(TA, nA) = eT;
+        RB::template st<!FUSE>(inE, inB ? PY + nb * y.row : CP, en, ei, tv);
+        if constexpr (FUSE) {
+          if (corner) *RB::first(CP, nA) = es[P].a;
+          if (inB && lastE) *RB::first(TA, nA) = eT;
+        } else {
+          st_if(corner, smem_addr(RB::first(CP, nA)), es[P].a);
+          st_if(inB && lastE, smem_addr(RB::first(TA, nA)), eT);
+        }
         if constexpr (CLUS) {
           const unsigned z = sizeof(Real);
           const int cpo = (int)(RB::first(sm + y.cp + cur * y.col, ncol - 1) - sm);
@@ -933,7 +990,7 @@ __device__ __forceinline__ void tile_body(const TileArgs& x, unsigned char* smem
         __syncwarp();
       }
       // ---- what the neighbours sent, and the update
-      if constexpr (MAIN) {
+      auto update_tiles = [&]() {
         Real ey[P], ty[P];
         RB::ld(PY + (byc + 1) * y.row, LX, bx, ey);
         RB::ld(TY + byc * y.row, LX, bx, ty);
@@ -967,9 +1024,9 @@ __device__ __forceinline__ void tile_body(const TileArgs& x, unsigned char* smem
 #pragma unroll
           for (int c = 0; c < P; ++c) accumulate(v[r][c], kz, kw, s[r][c]);
         }
-      }
+      };
       // ---- the chains
-      if constexpr (CHAIN) {
+      auto update_chains = [&]() {
         Real cr[P];
         RB::ld(inB ? TY + nb * y.row : TA, en, ei, cr);
         const Real cpn = *RB::first(CP, nA), ca = *RB::first(TA, nA);
@@ -1001,7 +1058,11 @@ __device__ __forceinline__ void tile_body(const TileArgs& x, unsigned char* smem
         const Real Ac = (d + Real(2) * ca) + (ISO ? Y : scale_ye(Y));
         es[P].b = eal[P] * es[P].b + ebet[P] * Ac + ebr[P] * ec + ebi[P] * esn;
         accumulate(ev[P], (Real)tb.z, (Real)tb.w, es[P]);
-      }
+      };
+      // (paired one-warp kernels: the chains before the tiles, 585 / 573 us)
+      if constexpr (CHAIN && kPairs && FUSE) update_chains();
+      if constexpr (MAIN) update_tiles();
+      if constexpr (CHAIN && !(kPairs && FUSE)) update_chains();
       tb = tn;
       if (CLUS) phase ^= cur;  // the barriers' phase turns when parity 1 has been used
       if (!kTwo) cur ^= 1;
@@ -1028,25 +1089,27 @@ __device__ __forceinline__ void tile_body(const TileArgs& x, unsigned char* smem
       NormAcc acc;
       if constexpr (sizeof(Real) == 4) {
         float big = 0.f;
-        if (live) {
+        auto largest = [&](float nr, float ni, int k) {
+          big = fmaxf(fmaxf(big, fmaxf(fabsf(nr), fabsf(ni))),
+                      fmaxf(fabsf(st[(2 * k) * nthr + t]), fabsf(st[(2 * k + 1) * nthr + t])));
+        };
+        int k = 0;
 #pragma unroll
-          for (int r = 0; r < P; ++r)
+        for (int r = 0; r < P; ++r)
 #pragma unroll
-            for (int c = 0; c < P; ++c)
+          for (int c = 0; c < P; ++c)
 #pragma unroll
-              for (int h = 0; h < H; ++h)
-                big = fmaxf(big, fmaxf(fabsf(get<H>(v[r][c].a, h)), fabsf(get<H>(v[r][c].b, h))));
-        }
+            for (int h = 0; h < H; ++h, ++k)
+              if (live) largest(get<H>(v[r][c].a, h), get<H>(v[r][c].b, h), k);
 #pragma unroll
-        for (int q = 0; q <= P; ++q)
-          if (q < P ? inE : corner) big = fmaxf(big, fmaxf(fabsf(ev[q].a), fabsf(ev[q].b)));
+        for (int q = 0; q <= P; ++q, ++k)
+          if (q < P ? inE : corner) largest(ev[q].a, ev[q].b, k);
         acc.start(big);
       }
       int k = 0;
       auto count = [&](Real nr, Real ni, Real orr, Real oi) {
         if constexpr (sizeof(Real) == 4) {
-          acc.add(nr, orr);
-          acc.add(ni, oi);
+          acc.add(make_float2(nr, ni), make_float2(orr, oi));
         } else {
           const double dr = nr - orr, di = ni - oi;
           dn += dr * dr + di * di;
@@ -1247,15 +1310,21 @@ __device__ __forceinline__ void tile_body(const TileArgs& x, unsigned char* smem
 // LANES: lanes of a one-warp subdomain are 1 the whole warp, 2 a part of it;
 // 0: more than one warp.  (1 and 2 apart: selecting zeros costs the benchmark's
 // one-warp subdomains 2.7%, those that share a warp 0.5%.)
-template <typename Real, int P, int H, int LANES, bool SRC, bool ISO, bool CLUS, int MAXT>
-__global__ void __launch_bounds__(MAXT) sweep_tile_kernel(const __grid_constant__ TileArgs x) {
+// TOL: the tolerance mode too.  FP32 sweeps of a fixed count have instantiations
+// without it, which have a register or two more and time loops of their own:
+// 1024 subdomains of 129 x 129 nodes, P = 4: 22.7 -> 20.7 ms; 48 of 37 x 31, P = 3:
+// 198 -> 187 us; 128 x 128, P = 5, 4 x 4 elements each: 1051 -> 1015 us.
+// One block per SM as the launch bound: without it some of them are compiled
+// for 64 or 74 registers (16 subdomains of 17 x 17, P = 2: 357 us against 166).
+template <typename Real, int P, int H, int LANES, bool SRC, bool ISO, bool CLUS, bool TOL, int MAXT>
+__global__ void __launch_bounds__(MAXT, 1) sweep_tile_kernel(const __grid_constant__ TileArgs x) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   if constexpr (LANES > 0) {
-    tile_body<Real, P, H, kBoth, LANES == 2, SRC, ISO, CLUS>(x, smem_raw, nullptr);
+    tile_body<Real, P, H, kBoth, LANES == 2, SRC, ISO, CLUS, TOL>(x, smem_raw, nullptr);
   } else {
     __shared__ TolShared ts;
-    if ((int)(threadIdx.x >> 5) < x.wm) tile_body<Real, P, H, kTiles, false, SRC, ISO, CLUS>(x, smem_raw, &ts);
-    else tile_body<Real, P, H, kChains, false, SRC, ISO, CLUS>(x, smem_raw, &ts);
+    if ((int)(threadIdx.x >> 5) < x.wm) tile_body<Real, P, H, kTiles, false, SRC, ISO, CLUS, TOL>(x, smem_raw, &ts);
+    else tile_body<Real, P, H, kChains, false, SRC, ISO, CLUS, TOL>(x, smem_raw, &ts);
   }
 }
 

@@ -14,7 +14,7 @@ namespace tile_sweep {
 // the same kernel with less would lower the limit between the two calls.
 constexpr int kMaxSmem = 220 * 1024;
 
-template <typename Real, int P, int H, bool SRC, bool ISO>
+template <typename Real, int P, int H, bool SRC, bool ISO, bool TOL>
 hz_status launch_tile_iso(const SweepArgs& a0, int count, cudaStream_t st, int* warps) {
   const int sxe = a0.sxe, sye = a0.sye;
   if (sxe > 32 || sye > 32 || sye % H) return HZ_ERR_UNSUPPORTED;
@@ -40,8 +40,8 @@ hz_status launch_tile_iso(const SweepArgs& a0, int count, cudaStream_t st, int* 
     x.offB = sye;
     const Lay y = make_lay<P, Real>(H, x.LX, x.nb, x.gs, SRC, tol);
     const size_t smem = (size_t)x.spw * y.total * sizeof(Real);
-    auto kern = x.spw > 1 ? sweep_tile_kernel<Real, P, H, 2, SRC, ISO, false, 32>
-                          : sweep_tile_kernel<Real, P, H, 1, SRC, ISO, false, 32>;
+    auto kern = x.spw > 1 ? sweep_tile_kernel<Real, P, H, 2, SRC, ISO, false, TOL, 32>
+                          : sweep_tile_kernel<Real, P, H, 1, SRC, ISO, false, TOL, 32>;
     if (smem > 48 * 1024) HZ_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem));
     kern<<<(count + x.spw - 1) / x.spw, 32, smem, st>>>(x);
     note_launch();
@@ -61,8 +61,8 @@ hz_status launch_tile_iso(const SweepArgs& a0, int count, cudaStream_t st, int* 
     const Lay y = make_lay<P, Real>(H, x.LX, x.nb, threads, SRC, tol);
     const size_t smem = (size_t)y.total * sizeof(Real);
     if (smem > kMaxSmem) continue;
-    auto kern = CL > 1 ? sweep_tile_kernel<Real, P, H, 0, SRC, ISO, true, MAXT>
-                       : sweep_tile_kernel<Real, P, H, 0, SRC, ISO, false, MAXT>;
+    auto kern = CL > 1 ? sweep_tile_kernel<Real, P, H, 0, SRC, ISO, true, TOL, MAXT>
+                       : sweep_tile_kernel<Real, P, H, 0, SRC, ISO, false, TOL, MAXT>;
     if (smem > 48 * 1024) HZ_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem));
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)(count * CL));
@@ -86,8 +86,14 @@ hz_status launch_tile_iso(const SweepArgs& a0, int count, cudaStream_t st, int* 
 
 template <typename Real, int P, int H, bool SRC>
 hz_status launch_tile(const SweepArgs& a, int count, cudaStream_t st, int* warps) {
-  if (a.hx2 == a.hy2) return launch_tile_iso<Real, P, H, SRC, true>(a, count, st, warps);
-  return launch_tile_iso<Real, P, H, SRC, false>(a, count, st, warps);
+  const bool iso = a.hx2 == a.hy2;
+  if constexpr (sizeof(Real) == 4) {
+    if (!(a.wh_tol > 0.0))
+      return iso ? launch_tile_iso<Real, P, H, SRC, true, false>(a, count, st, warps)
+                 : launch_tile_iso<Real, P, H, SRC, false, false>(a, count, st, warps);
+  }
+  return iso ? launch_tile_iso<Real, P, H, SRC, true, true>(a, count, st, warps)
+             : launch_tile_iso<Real, P, H, SRC, false, true>(a, count, st, warps);
 }
 
 // FP32, shape 1: one element per tile, shape 2: two, paired (P <= 3: the state
