@@ -57,7 +57,7 @@ extern "C" hz_status hz_solve_batch(const hz_problem* problems, int32_t count, c
     std::vector<std::string> seen;
     for (auto& [c, k] : order) {
       Problem& pr = *problems[k];
-      const std::string key = tune_key(pr.g, o.precision);
+      const std::string key = tune_key(pr, o.precision);
       if (std::find(seen.begin(), seen.end(), key) != seen.end()) continue;
       seen.push_back(key);
       HZ_CUDA(cudaSetDevice(pr.device));

@@ -80,9 +80,14 @@ struct Choice {
   int ty;       // block kernel: rows per thread (0 = by size, 1 = P, 2 = 2P);
                 // register-resident kernel: warps per subdomain (0/1, 2, 4)
 };
-std::string tune_key(const Geom& g, int precision);
-bool lookup_choice(const std::string& key, Choice* out);
-void store_choice(const std::string& key, Choice c);
+// What the autotuner keeps for a shape: the fastest kernel, and the fastest of
+// those that read a start (the register-resident and the block kernels).
+struct Tuned {
+  Choice best, warm;
+};
+std::string tune_key(const Problem& pr, int precision);
+bool lookup_tuned(const std::string& key, Tuned* out);
+void store_tuned(const std::string& key, const Tuned& c);
 hz_status autotune(Problem& pr, int precision, int nt, int m_wh, cudaStream_t st);
 int choose_nt(const Problem& pr, double cfl);
 hz_status prepare(Problem& pr, int nt, cudaStream_t st);

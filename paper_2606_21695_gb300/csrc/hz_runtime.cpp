@@ -241,17 +241,20 @@ void warp_rows(const Geom& g, WarpSweepArgs* w) {
 // ---- sweep kernel choices and the autotuner's cache
 namespace {
 std::mutex g_tune_mu;
-std::map<std::string, Choice> g_tuned;
+std::map<std::string, Tuned> g_tuned;
 }  // namespace
 
-std::string tune_key(const Geom& g, int precision) {
+std::string tune_key(const Problem& pr, int precision) {
+  const Geom& g = pr.g;
   int lb = 0;
   while ((1 << (lb + 1)) <= g.L) ++lb;  // occupancy depends on the number of subdomains
   return std::to_string(g.P) + "/" + std::to_string(g.nlx) + "x" + std::to_string(g.nly) + "/L2^" +
-         std::to_string(lb) + "/" + std::to_string(precision);
+         std::to_string(lb) + "/" + std::to_string(precision) +
+         (g.hx == g.hy ? "" : "/rect") +         // the element tiles have kernels of their own for square elements
+         (pr.robin_eta != 0.0 ? "/eta" : "");    // and none with interface boundary mass
 }
 
-bool lookup_choice(const std::string& key, Choice* out) {
+bool lookup_tuned(const std::string& key, Tuned* out) {
   std::lock_guard<std::mutex> lk(g_tune_mu);
   auto it = g_tuned.find(key);
   if (it == g_tuned.end()) return false;
@@ -259,7 +262,7 @@ bool lookup_choice(const std::string& key, Choice* out) {
   return true;
 }
 
-void store_choice(const std::string& key, Choice c) {
+void store_tuned(const std::string& key, const Tuned& c) {
   std::lock_guard<std::mutex> lk(g_tune_mu);
   g_tuned[key] = c;
 }
@@ -366,11 +369,11 @@ std::mutex g_tune_run_mu;
 // tiles of one or two elements; warp per subdomain; one block per subdomain
 // with P or 2P rows per thread; a cluster of blocks) on this problem and caches the fastest per shape key.
 hz_status autotune(Problem& pr, int precision, int nt, int m_wh, cudaStream_t st) {
-  const std::string key = tune_key(pr.g, precision);
-  Choice c{};
-  if (lookup_choice(key, &c)) return HZ_OK;
+  const std::string key = tune_key(pr, precision);
+  Tuned c{};
+  if (lookup_tuned(key, &c)) return HZ_OK;
   std::lock_guard<std::mutex> lk(g_tune_run_mu);
-  if (lookup_choice(key, &c)) return HZ_OK;
+  if (lookup_tuned(key, &c)) return HZ_OK;
   HZ_TRY(prepare(pr, nt, st));
   HZ_TRY(ensure_flags(pr));
   const size_t vb = (size_t)pr.g.lam_complex() * 2 * sizeof(double);
@@ -387,8 +390,8 @@ hz_status autotune(Problem& pr, int precision, int nt, int m_wh, cudaStream_t st
   cudaEvent_t e0, e1;
   HZ_CUDA(cudaEventCreate(&e0));
   HZ_CUDA(cudaEventCreate(&e1));
-  float best = 1e30f;
-  Choice bc{kVariantBlock, 0};
+  float best = 1e30f, best_warm = 1e30f;
+  Choice bc{kVariantBlock, 0}, wc{kVariantBlock, 0};
   for (const Choice& cand : cands) {
     hz_status s = launch_choice(pr, a, cand, fp32, st);  // warm-up, also the support check
     if (s == HZ_ERR_UNSUPPORTED) continue;
@@ -410,11 +413,15 @@ hz_status autotune(Problem& pr, int precision, int nt, int m_wh, cudaStream_t st
       best = ms;
       bc = cand;
     }
+    if ((cand.variant == kVariantWarp || cand.variant == kVariantBlock) && ms < best_warm) {
+      best_warm = ms;
+      wc = cand;
+    }
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   HZ_CUDA(cudaGetLastError());
-  store_choice(key, bc);
+  store_tuned(key, {bc, wc});
   if (std::getenv("HZ_TUNE_LOG"))
     std::fprintf(stderr, "hz autotune %s: variant %d/%d, %.4f ms per sweep\n", key.c_str(), bc.variant, bc.ty, best / 2);
   return HZ_OK;
@@ -507,12 +514,12 @@ hz_status sweep(Problem& pr, int precision, int nt, int m_wh, double wh_tol, con
   if (u0) {
     a.u0 = u0;
     hz_status ws = HZ_ERR_UNSUPPORTED;
-    // the kernel the autotuner chose for this shape when it reads the start
+    // the autotuner's fastest kernel among those that read the start
     // (register-resident 1/2/4 warps or block), HZ_SWEEP_WARPS forcing the
     // register-resident shape (tests); else one warp, else the block kernel
-    Choice tc{};
-    const bool tuned = pr.autotune && lookup_choice(tune_key(pr.g, precision), &tc) &&
-                       (tc.variant == kVariantWarp || tc.variant == kVariantBlock);
+    Tuned kept{};
+    const bool tuned = pr.autotune && lookup_tuned(tune_key(pr, precision), &kept);
+    const Choice tc = kept.warm;
     const char* hw = std::getenv("HZ_SWEEP_WARPS");
     if (fp32 && !trial && (hw || (tuned && tc.variant == kVariantWarp) || !tuned)) {
       const int h = hw ? std::atoi(hw) : (tuned ? tc.ty : 1);
@@ -533,10 +540,9 @@ hz_status sweep(Problem& pr, int precision, int nt, int m_wh, double wh_tol, con
     return HZ_OK;
   }
   const int want = trial ? kVariantBlock : sweep_variant();  // 16-bit trials run on the block kernel
-  Choice ch{};
-  bool have = false;
-  if (want == kVariantAuto && pr.autotune && lookup_choice(tune_key(pr.g, precision), &ch)) have = true;
-  (void)trial;
+  Tuned kept{};
+  const bool have = want == kVariantAuto && pr.autotune && lookup_tuned(tune_key(pr, precision), &kept);
+  const Choice ch = kept.best;
   hz_status ls = HZ_ERR_UNSUPPORTED;
   if (have) {
     ls = launch_choice(pr, a, ch, fp32, st);
