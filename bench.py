@@ -42,11 +42,25 @@ if ROOT not in sys.path:
 
 METRIC = "DOF-updates/s"
 UNIT = "DOF-updates/s"
-# DRAM bytes (read + write) of one launch of the one-warp-per-subdomain sweep
-# on the 256x256, P=3 workload, from one ncu capture of this kernel version
+# DRAM bytes (read + write) of one launch of the element-tile sweep (paired
+# tiles, one warp per subdomain) on the 256x256, P=3 workload, from one ncu capture
 # (coefficients and lambda read once; independent of the WaveHoltz count)
-SWEEP_WARP_TRAFFIC_BYTES = 7.604480e6
+SWEEP_TILE_TRAFFIC_BYTES = 7.604480e6
 TOL = 1e-8
+
+
+def sweep_kernel_name(report):
+    """The sweep kernel of a solve report: element tiles report 32 x elements per tile + warps as their shape."""
+    v, shape = report["sweep_variant"], report["sweep_shape"]
+    tiles, warps = divmod(shape, 32)
+    if v == 6:
+        return "sweep_mapped_tile_kernel (element per thread)" if tiles else "sweep_mapped_kernel (node per thread)"
+    if v in (2, 5) and tiles:
+        where = f"{warps} warp(s) per subdomain" if v == 2 else "a cluster per subdomain"
+        return f"sweep_tile_kernel ({tiles} element(s) per tile, {where})"
+    return {1: "sweep_kernel (block)", 2: f"sweep_band_kernel ({shape} warps per subdomain)" if shape > 1
+            else "sweep_warp_kernel (one warp per subdomain)", 3: "sweep_cluster_kernel", 4: "sweep_packed_kernel",
+            5: "sweep_cband_kernel"}.get(v, "?")
 
 
 def parse():
@@ -803,21 +817,16 @@ def run_ours(args):
             "peaks": peaks,
             "fp64_solve": fp64,
             "solve": {"sweeps_per_solve": sweeps / args.steps, "rel_residual_max": max(res),
-                      "sweep_kernel": {1: "block", 2: "warps (element tiles or node columns)", 3: "cluster", 4: "packed",
-                                       5: "cluster of warps", 6: "mapped (element form)"}.get(reports[0]["sweep_variant"]),
+                      "sweep_kernel": sweep_kernel_name(reports[0]),
                       "refinements": reports[0]["refinements"], "gmres_iters": reports[0]["gmres_iters"],
                       "dof_updates_per_solve": dof / args.steps},
-            "roofline": {"kernel": {1: "sweep_kernel (block)",
-                                    2: ("sweep_tile_kernel (element tiles) or a node-column kernel, "
-                                        f"{max(reports[0]['sweep_shape'], 1)} warp(s) per subdomain"),
-                                    3: "sweep_cluster_kernel", 5: "sweep_tile_kernel or sweep_cband_kernel on clusters",
-                                    6: "sweep_mapped_kernel (element form, block per subdomain)"}.get(reports[0]["sweep_variant"], "?")
+            "roofline": {"kernel": sweep_kernel_name(reports[0])
                          + " FP32, one launch = one DD sweep", "bound": "alu",
                          "achieved": achieved, "peak": peaks["fp32_tflops"], "unit": "TFLOP/s",
                          "frac": achieved / peaks["fp32_tflops"],
                          "peak_source": "measured in this run (hz_fma_peak, FP32 FMA)",
-                         "traffic": SWEEP_WARP_TRAFFIC_BYTES if (wl.P == 3 and reports[0]["sweep_variant"] == 2
-                                                                 and reports[0]["sweep_shape"] == 1) else None,
+                         "traffic": SWEEP_TILE_TRAFFIC_BYTES if (wl.P == 3 and reports[0]["sweep_variant"] == 2
+                                                                 and reports[0]["sweep_shape"] == 65) else None,
                          "traffic_unit": "bytes per launch (DRAM, ncu)",
                          "sweep_shape": reports[0]["sweep_shape"],
                          "algorithmic": f"{flops_per_update:.4g} flop/DOF-update x {dof_per_launch:.4g} DOF-updates/launch",

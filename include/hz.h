@@ -178,7 +178,8 @@ typedef struct {
                             node columns), 3 cluster, 4 packed with other solves, 5 cluster of warps
                             (element tiles or bands), 6 mapped mesh */
   int32_t sweep_shape;   /* its configuration: warps per subdomain (2), rows per thread in units
-                            of the degree (1, 3; 0 = chosen by size) */
+                            of the degree (1, 3; 0 = chosen by size); element tiles (2, 5, 6):
+                            32 x elements per tile + warps per subdomain (5, 6: 32 x elements) */
   double sweep_seconds;  /* device time of the sweep kernels (CUDA events on the solve's stream) */
 } hz_solve_report;
 

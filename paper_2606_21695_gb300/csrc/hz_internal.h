@@ -152,8 +152,8 @@ hz_status launch_sweep_cband(int P, const SweepArgs& a, int L, cudaStream_t st);
 // elements, degree 1..5 (FP64: 1..4), eta = 0, cold start.
 // a.ty_force: 1 = one element per tile, 2 = two, paired (FP32, P <= 3, even
 // sub_ny), 0 = by size (tile_shape).  *warps: warps per subdomain, 0 for a
-// cluster.  HZ_ERR_UNSUPPORTED (nothing launched) else.
-hz_status launch_sweep_tile(bool fp32, int P, const SweepArgs& a, int count, cudaStream_t st, int* warps);
+// cluster.  *elements: elements per tile.  HZ_ERR_UNSUPPORTED (nothing launched) else.
+hz_status launch_sweep_tile(bool fp32, int P, const SweepArgs& a, int count, cudaStream_t st, int* warps, int* elements);
 // Shape of the tile sweep for a subdomain (1 or 2), and whether it is the
 // default kernel there (without the autotuner).  L: subdomains of the problem.
 int tile_shape(bool fp32, int P, int sxe, int sye, int L);

@@ -72,6 +72,9 @@ struct hz_problem_s {
 
 namespace hz {
 using Problem = hz_problem_s;
+// Configurations of the element tiles, Cartesian or curved, are reported as
+// kTileShape x elements per tile + warps per subdomain (0: a cluster).
+constexpr int kTileShape = 32;
 constexpr int kVariantAuto = 0, kVariantBlock = 1, kVariantWarp = 2, kVariantCluster = 3, kVariantPacked = 4,
               kVariantClusterBand = 5, kVariantMapped = 6, kVariantTile = 7;
 int sweep_variant();

@@ -272,13 +272,13 @@ hz_status launch_choice(Problem& pr, const SweepArgs& a0, Choice c, bool fp32, c
   const int count = sweep_count(a0, g.L);
   hz_status s = HZ_ERR_UNSUPPORTED;
   if (c.variant == kVariantTile) {
-    int warps = 0;
+    int warps = 0, elements = 0;
     SweepArgs a = a0;
     a.ty_force = c.ty;  // elements per tile: 1, 2 or 0 = by size
-    s = launch_sweep_tile(fp32, g.P, a, count, st, &warps);
+    s = launch_sweep_tile(fp32, g.P, a, count, st, &warps, &elements);
     if (s == HZ_OK) {  // reported with the register-resident kernels by warps per subdomain, or as a cluster
       pr.last_variant = warps > 0 ? kVariantWarp : kVariantClusterBand;
-      pr.last_shape = warps;
+      pr.last_shape = kTileShape * elements + warps;
     }
     return s;
   }
@@ -459,7 +459,7 @@ hz_status sweep(Problem& pr, int precision, int nt, int m_wh, double wh_tol, con
     pr.ev_used += 2;
     HZ_CUDA(cudaEventRecord(e0, st));
   }
-  // general convex quadrilaterals: the element-form kernel (one variant)
+  // general convex quadrilaterals: the element-form kernels (a thread per element or per node)
   if (pr.mapped) {
     if (trial) return fail(HZ_ERR_UNSUPPORTED, "16-bit trials are not built for mapped meshes");
     MappedSweepArgs ma{};
@@ -478,9 +478,10 @@ hz_status sweep(Problem& pr, int precision, int nt, int m_wh, double wh_tol, con
       ms = launch_sweep_mapped_tile(g.P, ma, count, st);
       if (ms != HZ_OK && (ms != HZ_ERR_UNSUPPORTED || mv == kVariantTile)) return ms;
     }
-    if (ms != HZ_OK) HZ_TRY(launch_sweep_mapped(fp32, g.P, ma, count, st));
+    const bool tiles = ms == HZ_OK;
+    if (!tiles) HZ_TRY(launch_sweep_mapped(fp32, g.P, ma, count, st));
     pr.last_variant = kVariantMapped;
-    pr.last_shape = 0;
+    pr.last_shape = tiles ? kTileShape : 0;
     if (e1) HZ_CUDA(cudaEventRecord(e1, st));
     pr.sweeps_launched++;
     return HZ_OK;

@@ -70,7 +70,7 @@ bool tile_default(bool fp32, int P, int sxe, int sye, int L) {
   return true;
 }
 
-hz_status launch_sweep_tile(bool fp32, int P, const SweepArgs& a, int count, cudaStream_t st, int* warps) {
+hz_status launch_sweep_tile(bool fp32, int P, const SweepArgs& a, int count, cudaStream_t st, int* warps, int* elements) {
   if (a.round_mode != 0 || a.eta != 0.0 || a.u0) return HZ_ERR_UNSUPPORTED;
   if (a.sxe > 32 || a.sye > 32) return HZ_ERR_UNSUPPORTED;
   int shape = a.ty_force;
@@ -79,6 +79,7 @@ hz_status launch_sweep_tile(bool fp32, int P, const SweepArgs& a, int count, cud
     shape = v ? std::atoi(v) : tile_shape(fp32, P, a.sxe, a.sye, a.Sx * a.Sy);
   }
   if (shape == 2 && (!fp32 || P > 3 || a.sye % 2)) return HZ_ERR_UNSUPPORTED;
+  *elements = shape == 2 ? 2 : 1;
   if (fp32) {
     switch (P) {
       case 1: return tile_sweep::tile_f32_p1(shape, a, count, st, warps);

@@ -1,5 +1,6 @@
 """Sweep kernels that the size rules no longer take by themselves, and shapes of the element tiles that other tests reach
-only with non-square elements or with a source, against the FP64 oracle (the bounds of tests/_tolerances.py)."""
+only with non-square elements or with a source, against the FP64 oracle (the bounds of tests/_tolerances.py).  Also that
+a solve's report tells the kernels apart."""
 
 import numpy as np
 import pytest
@@ -83,3 +84,16 @@ def test_warm_start_on_curved_tiles(hz, monkeypatch, nx, ny, sx, sy, P):
     assert _rel(_host_c(u).reshape(ref_u.shape), ref_u) < FP32_REL
     assert _rel(_host_c(lout).reshape(ref_l.shape), ref_l) < FP32_REL
     case.close()
+
+
+def test_reports_tell_the_kernels_apart(hz, monkeypatch):
+    seen = {}
+    for env in ("tile1", "tile2", "warp", "block"):
+        monkeypatch.setenv("HZ_SWEEP_VARIANT", env[:4] if env.startswith("tile") else env)
+        monkeypatch.setenv("HZ_TILE_SHAPE", env[4:] or "0")
+        case, _ = _pair(hz, _wl(16, 16, 8, 8, 3))
+        _, _, rep = hz.hz_solve(case.pr, hz.hz_default_opts(precision=hz.HZ_FP32_REFINE, tol=1e-4), n=case.n)
+        seen[env] = rep["sweep_variant"], rep["sweep_shape"]
+        case.close()
+    assert seen["tile1"] == (2, 32 + 3) and seen["tile2"] == (2, 64 + 1)
+    assert seen["warp"] == (2, 1) and seen["block"][0] == 1
