@@ -8,7 +8,8 @@ namespace hz {
 // One thread per element runs (P+1)^2 nodes in a row, the other kernel one
 // node per thread: the tiles win once the node kernel's blocks fill the SMs
 // (about 900 of its threads an SM) or need more than one pass over a block.
-// Node kernel / tiles, 5 WaveHoltz iterations: P = 3, 8 x 8 elements: 196 / 119
+// Node kernel / tiles, 5 WaveHoltz iterations at 14 node spacings per wavelength
+// (N_t about a third above that of square elements): P = 3, 8 x 8 elements: 196 / 119
 // us at 9 subdomains, 388 / 127 at 256, 1343 / 349 at 1024; P = 3, 4 x 4: 106 /
 // 130 at 256, 270 / 135 at 1024; P = 4, 4 x 4: 231 / 324 at 256, 809 / 330 at
 // 1024; P = 2, 16 x 12: 338 / 102 at 9.  Tiles that leave half of the lanes

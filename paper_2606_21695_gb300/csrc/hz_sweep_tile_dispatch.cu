@@ -24,8 +24,9 @@ int one_element_lanes(int sxe, int sye) { return tile_pow2(sxe) * sye; }
 
 // Two paired elements per tile halve the instructions per node (packed FMAs)
 // but leave half the warps: better once one-element tiles fill the SMs'
-// resident blocks.  Sweeps of 5 WaveHoltz iterations, one / two elements:
-// P = 3, 8 x 8 elements: 40 / 62 us at 9 subdomains, 57 / 63 at 256, 69 / 64 at
+// resident blocks.  Sweeps of 5 WaveHoltz iterations at 14 node spacings per
+// wavelength (N_t = 21, 24, 32, 38 and 44 for P = 1 to 5; all timings of this file, taken before
+// fixed-count sweeps had kernels of their own), one / two elements: P = 3, 8 x 8 elements: 40 / 62 us at 9 subdomains, 57 / 63 at 256, 69 / 64 at
 // 576, 131 / 104 at 1024; P = 2, 16 x 16: 73 / 55 at 256; P = 3, 32 x 32: 103 /
 // 157 at 9, 202 / 157 at 64.  Degrees 1 and 2 gain earlier (P = 2, 12 x 10: 36 /
 // 29 at 9, 16 x 16: 38 / 37); P = 4 loses (see launch_tile_f32), and P = 3 where
@@ -55,7 +56,8 @@ int tile_shape(bool fp32, int P, int sxe, int sye, int L) {
 //    at 64, 155 / 178 at 576, 250 / 180 at 1024).
 // FP64 (bound by the FP64 pipe; 3 iterations): with a subdomain per SM and
 // whole tiles (P = 3, 8 x 8 at 256: 915 / 648, at 64: 466 / 501; P = 4,
-// 16 x 16 at 16: 2364 / 1458; P = 3, 32 x 32 at 64: 3905 / 2354).
+// 16 x 16 at 16: 2364 / 1458; P = 3, 32 x 32 at 64: 3905 / 2354).  P = 2 and other
+// sye were not timed by themselves: the limits are those of whole tiles per warp.
 bool tile_default(bool fp32, int P, int sxe, int sye, int L) {
   if (sxe > 32 || sye > 32 || P > (fp32 ? 5 : 4)) return false;
   const int lanes = one_element_lanes(sxe, sye), sms = sm_count();

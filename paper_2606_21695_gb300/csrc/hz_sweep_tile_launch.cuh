@@ -97,7 +97,7 @@ hz_status launch_tile(const SweepArgs& a, int count, cudaStream_t st, int* warps
 }
 
 // FP32, shape 1: one element per tile, shape 2: two, paired (P <= 3: the state
-// of two larger elements leaves too few warps; P = 4, 8 x 8 elements at 1024
+// of two larger elements leaves too few warps; P = 4, N_t = 38, 8 x 8 elements at 1024
 // subdomains: 235 us one by one, 241 paired, 16 x 16 at 256: 239, 264).
 template <int P>
 hz_status launch_tile_f32(int shape, const SweepArgs& a, int count, cudaStream_t st, int* warps) {
